@@ -96,7 +96,7 @@ bool batch_eligible(const Plan *const *plans, int n) {
     int groups = 0;
     for (int i = 0; i < n; i++) {
         const Plan &P = *plans[i];
-        if (P.prec != FMM_PREC_MIXED || P.step != 1 || !P.Mf || P.m2l_tc || !P.f32_tab || !P.box_geo || !P.box_cf) return false;
+        if (P.prec != FMM_PREC_MIXED || P.step != 1 || !P.Mf || P.m2l_tc || !m2l_f32_supported(P.p) || !P.box_geo || !P.box_cf) return false;
         if (P.dtype != A.dtype || P.device != A.device) return false;
         if (!seen[P.p]) seen[P.p] = true, groups++;
     }

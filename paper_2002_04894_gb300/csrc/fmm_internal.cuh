@@ -231,10 +231,11 @@ inline void stage_mark(Plan &P, int stage, int edge) {
 // Device helpers
 // ---------------------------------------------------------------------------
 __host__ __device__ inline int tri(int n, int m) { return n * (n + 1) / 2 + m; }
-__host__ __device__ inline int ncoef(int p) { return (p + 1) * (p + 2) / 2; }
-// row stride (coefficients) of the float multipoles Mf: even, so that
-// coefficient pairs (2i, 2i+1) are 16-byte aligned
-__host__ __device__ inline int mf_stride(int p) { return (ncoef(p) + 1) & ~1; }
+__host__ __device__ constexpr int ncoef(int p) { return (p + 1) * (p + 2) / 2; }
+// row stride (coefficients) of the float multipoles Mf: an odd number of
+// 16-byte pieces, so that coefficient pairs (2i, 2i+1) are aligned and rows
+// copied to shared memory as they stand are read without bank conflicts
+__host__ __device__ constexpr int mf_stride(int p) { return 2 * (((ncoef(p) + 1) / 2) | 1); }
 
 // Order-preserving map from doubles to unsigned 64-bit keys (no NaN; -0 was
 // canonicalised to +0 on input).

@@ -35,6 +35,7 @@
 
 #include "fmm_internal.cuh"
 #include "m2l_common.cuh"
+#include "m2l_reg.cuh"
 
 namespace fmm {
 
@@ -1260,8 +1261,10 @@ cudaError_t m2l_all(Plan &P) {
 // with r_s/rho, r_t/rho < 1 for every weak pair: all float values stay O(1).
 // The target's local expansion is accumulated in double.
 //
-// GPU mapping: one weak pair per thread, all levels in one launch (pairs
-// sorted by target), blocks striding over chunks of 128 pairs. Every degree
+// Orders 1..12 keep the pair in registers (m2l_reg.cuh). GPU mapping of
+// orders 14 and 16, whose pair does not fit: one weak pair per thread, all
+// levels in one launch (pairs sorted by target), blocks striding over chunks
+// of 128 pairs. Every degree
 // (and every two orders of the translation) is its own template instance,
 // so a degree's input vector sits in registers; a fold's outputs come from a
 // runtime loop, two per iteration (one of each parity), each a dot product
@@ -1304,10 +1307,8 @@ __device__ __forceinline__ float2 fmulc(float2 a, float2 b) {
 // Per-pair coefficient storage between the stages: degrees 0..kTmDeg live
 // in the thread's lane of tensor memory (Re, Im interleaved: columns
 // 2 tri(n,m), 2 tri(n,m)+1), the rest in a shared-memory column of the
-// block (stride T). Tensor memory is otherwise idle in this kernel; moving
-// 55 of the 91 coefficients (p = 12) there cuts shared memory per block from
-// 111 to 55 KB, so three blocks (12 warps, register-limited) fit an SM
-// instead of two.
+// block (stride T). Tensor memory is otherwise idle in this kernel, and 55
+// of the coefficients there leave shared memory for more resident blocks.
 constexpr int kTmDeg = 9;
 constexpr int kTmC = (kTmDeg + 1) * (kTmDeg + 2) / 2;  // first coefficient in shared memory
 
@@ -2032,15 +2033,35 @@ cudaError_t launch_f32(Plan &Pl, int64_t tot) {
 
 }  // namespace
 
-bool m2l_f32_supported(int p) {
-    return p == 4 || p == 6 || p == 8 || p == 10 || p == 12 || p == 14 || p == 16;
+namespace reg {
+FMM_M2L_REG(extern, 1) FMM_M2L_REG(extern, 2) FMM_M2L_REG(extern, 3) FMM_M2L_REG(extern, 4)
+FMM_M2L_REG(extern, 5) FMM_M2L_REG(extern, 6) FMM_M2L_REG(extern, 7) FMM_M2L_REG(extern, 8)
+FMM_M2L_REG(extern, 9) FMM_M2L_REG(extern, 10) FMM_M2L_REG(extern, 11) FMM_M2L_REG(extern, 12)
+}  // namespace reg
+
+// f(integral_constant<P>) for the order p of a register-resident instance
+template <typename F>
+static cudaError_t with_reg_order(int p, F &&f) {
+    switch (p) {
+#define FMM_CASE(P) \
+    case P: return f(std::integral_constant<int, P>{});
+        FMM_CASE(1) FMM_CASE(2) FMM_CASE(3) FMM_CASE(4) FMM_CASE(5) FMM_CASE(6)
+        FMM_CASE(7) FMM_CASE(8) FMM_CASE(9) FMM_CASE(10) FMM_CASE(11) FMM_CASE(12)
+#undef FMM_CASE
+        default: return cudaErrorInvalidValue;
+    }
 }
+
+// Orders whose pair fits a thread's registers run m2l_reg.cuh; 14 and 16 keep
+// the pair in tensor and shared memory (k_m2l_rot_f32); the other orders take
+// the FP64 M2L.
+static bool m2l_in_registers(int p) { return p >= 1 && p <= 12; }
+bool m2l_f32_supported(int p) { return m2l_in_registers(p) || p == 14 || p == 16; }
 
 // plan-time setup, so that evaluations are safe to capture into a graph
 cudaError_t m2l_f32_setup(Plan &P) {
-    // the SIMT float kernel by default; the tensor-core kernel on request, and
-    // for orders without a SIMT instance
-    const bool tc = m2l_tc_supported(P.p) && (P.tc_m2l_opt || !m2l_f32_supported(P.p));
+    // the tensor-core kernel only on request
+    const bool tc = m2l_tc_supported(P.p) && P.tc_m2l_opt;
     if (!tc && !m2l_f32_supported(P.p)) return cudaSuccess;  // FP64 M2L
     P.Mf = (float2 *)palloc(P, (size_t)P.nbox * mf_stride(P.p) * sizeof(float2));
     P.Lh = (double2 *)palloc(P, (size_t)P.nbox * P.nc * sizeof(double2));
@@ -2049,6 +2070,8 @@ cudaError_t m2l_f32_setup(Plan &P) {
         P.m2l_tc = true;
         return m2l_tc_setup(P);
     }
+    if (m2l_in_registers(P.p))
+        return with_reg_order(P.p, [](auto o) { return reg::reg_attr<decltype(o)::value>(); });
     const std::vector<float4> &pt = f32_pair_tables_cached(P.p);
     P.f32_tab = palloc(P, pt.size() * sizeof(float4));
     if (!P.f32_tab) return cudaErrorMemoryAllocation;
@@ -2056,11 +2079,6 @@ cudaError_t m2l_f32_setup(Plan &P) {
     cudaError_t e = cudaMemcpyAsync(P.f32_tab, pt.data(), pt.size() * sizeof(float4), cudaMemcpyHostToDevice, P.stream);
     if (e != cudaSuccess) return e;
     switch (P.p) {
-        case 4: return attr_f32<4>();
-        case 6: return attr_f32<6>();
-        case 8: return attr_f32<8>();
-        case 10: return attr_f32<10>();
-        case 12: return attr_f32<12>();
         case 14: return attr_f32<14>();
         case 16: return attr_f32<16>();
         default: return cudaSuccess;
@@ -2077,13 +2095,14 @@ cudaError_t m2l_f32_all(Plan &P) {
     cudaError_t e = cudaSuccess;
     if (tot > 0 && P.m2l_tc) {
         e = m2l_tc_launch(P);
+    } else if (tot > 0 && m2l_in_registers(P.p)) {
+        const PairTable PT = pair_table(P);
+        e = with_reg_order(P.p, [&](auto o) {
+            reg::reg_launch<decltype(o)::value>(PT, tot, P.box_cf, P.Mf, P.Lh, P.d_err, P.stream);
+            return cudaGetLastError();
+        });
     } else if (tot > 0) {
         switch (P.p) {
-            case 4: e = launch_f32<4>(P, tot); break;
-            case 6: e = launch_f32<6>(P, tot); break;
-            case 8: e = launch_f32<8>(P, tot); break;
-            case 10: e = launch_f32<10>(P, tot); break;
-            case 12: e = launch_f32<12>(P, tot); break;
             case 14: e = launch_f32<14>(P, tot); break;
             case 16: e = launch_f32<16>(P, tot); break;
             default: return cudaErrorInvalidValue;
@@ -2106,12 +2125,12 @@ cudaError_t batch_m2m_up(const BatchSys *S, const int32_t *off, int nsys, int64_
 cudaError_t batch_m2l(const BatchSys *S, const int32_t *off, int nsys, int64_t nchunks, int p, const void *tab,
                       cudaStream_t st) {
     if (nchunks == 0) return cudaGetLastError();
+    if (m2l_in_registers(p))
+        return with_reg_order(p, [&](auto o) {
+            reg::reg_launch_batch<decltype(o)::value>(S, off, nsys, nchunks, st);
+            return cudaGetLastError();
+        });
     switch (p) {
-        case 4: launch_b_f32<4>(S, off, nsys, nchunks, tab, st); break;
-        case 6: launch_b_f32<6>(S, off, nsys, nchunks, tab, st); break;
-        case 8: launch_b_f32<8>(S, off, nsys, nchunks, tab, st); break;
-        case 10: launch_b_f32<10>(S, off, nsys, nchunks, tab, st); break;
-        case 12: launch_b_f32<12>(S, off, nsys, nchunks, tab, st); break;
         case 14: launch_b_f32<14>(S, off, nsys, nchunks, tab, st); break;
         case 16: launch_b_f32<16>(S, off, nsys, nchunks, tab, st); break;
         default: return cudaErrorInvalidValue;

@@ -1,0 +1,10 @@
+// Instances of the register-resident M2L (m2l_reg.cuh).
+#include "m2l_reg.cuh"
+
+namespace fmm {
+namespace reg {
+FMM_M2L_REG(, 10)
+FMM_M2L_REG(, 2)
+FMM_M2L_REG(, 3)
+}  // namespace reg
+}  // namespace fmm

@@ -1,0 +1,9 @@
+// Instances of the register-resident M2L (m2l_reg.cuh).
+#include "m2l_reg.cuh"
+
+namespace fmm {
+namespace reg {
+FMM_M2L_REG(, 5)
+FMM_M2L_REG(, 6)
+}  // namespace reg
+}  // namespace fmm

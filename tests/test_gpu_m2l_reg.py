@@ -1,0 +1,62 @@
+"""The register-resident single-precision M2L (orders 1..12, Sec. 2.1.3
+rotation form) against the FP64 M2L on the same points.
+
+Tolerance, from the operation count: five chained contractions of at most
+p + 1 terms in single precision (unit roundoff 2^-24), and the float P2M
+before them (sums of depth <= 16): the local expansions, every degree scaled to
+its box (L_k r^k), differ by at most (5 (p + 1) + 16) 2^-24 of their norm."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2002_04894_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+# kind, n, levels, theta: few pairs (part of one warp's 32), many short target runs, long lists, a ragged tail
+SIZES = [("uniform", 300, 4, 0.7), ("uniform", 700, 5, 0.7), ("plummer", 6000, 9, 0.5), ("gmm", 20000, 8, 0.6)]
+
+
+def scaled_locals(fmm, plan, p):
+    L = fmm.fmm_eval_expansions(plan, "L")
+    k = np.concatenate([np.full(n + 1, n) for n in range(p + 1)])
+    return L * fmm.fmm_plan_tree(plan)["radius"][:, None] ** k
+
+
+@pytest.mark.parametrize("p", range(1, 13))
+def test_locals_match_fp64(gpu_lib, p):
+    fmm = gpu_lib
+    for kind, n, levels, theta in SIZES:
+        x = torch.from_numpy(inputs.points(kind, n, seed=p)).cuda()
+        q = torch.from_numpy(inputs.charges_uniform(n, seed=p)).cuda()
+        got = []
+        for prec in (fmm.FMM_PREC_FP64, fmm.FMM_PREC_MIXED):
+            plan = fmm.fmm_plan(x, levels, p, theta, prec=prec)
+            fmm.fmm_eval(plan, q)
+            fmm.fmm_eval_check(plan)
+            assert fmm.fmm_plan_stats(plan)["weak_pairs"] > 0
+            got.append(scaled_locals(fmm, plan, p))
+        err = np.linalg.norm(got[1] - got[0]) / np.linalg.norm(got[0])
+        assert err <= (5 * (p + 1) + 16) * 2.0 ** -24, (kind, n, err)
+
+
+@pytest.mark.parametrize("p", [1, 5, 9, 11, 12])
+def test_batch_equals_alone(gpu_lib, p):
+    """Systems of different pair counts (none, part of a warp, ragged) in one batch."""
+    fmm = gpu_lib
+    plans, qs, pots, alone = [], [], [], []
+    for i, (kind, n, levels) in enumerate([("uniform", 40, 1), ("uniform", 700, 5), ("plummer", 9000, 7), ("gmm", 3000, 6)]):
+        x = torch.from_numpy(inputs.points(kind, n, seed=i).astype(np.float32)).cuda()
+        q = torch.from_numpy(inputs.charges_uniform(n, seed=i).astype(np.float32)).cuda()
+        plans.append(fmm.fmm_plan(x, levels, p, 0.6, prec=fmm.FMM_PREC_MIXED))
+        alone.append(fmm.fmm_eval(plans[-1], q)[0])
+        qs.append(q)
+        pots.append(torch.zeros(n, device="cuda"))
+    torch.cuda.synchronize()
+    batch = fmm.fmm_batch_create(plans, qs, pots)
+    assert fmm.fmm_batch_info(batch)["fused"]
+    fmm.fmm_batch_launch(batch)
+    for plan, a, b in zip(plans, alone, pots):
+        fmm.fmm_eval_check(plan)
+        # the same sums in another order of the double atomics: a float ulp or two (as the other batch tests hold)
+        assert float((a - b).norm() / a.norm()) <= 1e-6
