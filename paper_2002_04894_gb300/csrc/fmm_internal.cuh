@@ -20,6 +20,8 @@ constexpr int kP2PTileSmall = 64;
 // sources per near-field work unit at most (about): a target leaf whose
 // strong list holds more is cut into segments, each its own unit
 constexpr int kP2PSegSources = 1 << 16;
+// few leaves: units per SM to cut their lists for, and the shortest segment
+constexpr int kP2PUnitsPerSM = 10, kP2PSegMin = 256;
 
 // ---------------------------------------------------------------------------
 // Plan: everything lives in device memory owned by the plan.
@@ -79,6 +81,59 @@ __device__ __forceinline__ float offset_f(float ah, float bh, float al, float bl
 
 // 2^k as a double, for |k| <= 1022 (exact; integer operations only)
 __device__ __forceinline__ double pow2i(int k) { return __longlong_as_double((long long)(1023 + k) << 52); }
+
+// How the T threads of a near-field unit take its nt <= T targets. The first
+// nt - nt % 32 threads take a target each, against every source; the r =
+// nt % 32 targets left over share the remaining threads, `slices` to a
+// target, thread k of them taking sources slice, slice + slices, ... A warp
+// costs the same however few of its lanes have a target: with one target per
+// thread throughout, a leaf of 73 points left a quarter of the issued lanes
+// idle (300k points, 4096 leaves: near field 7.14 -> 5.64 ms; 100k points in
+// leaves of 24: 0.91 -> 0.53 ms; leaves of 61 or 122 points: no change).
+struct P2PLane {
+    int target, slice, slices, rest;  // rest: threads with slices of the left-over targets, in all
+    bool active;
+    int first, left;  // the left-over targets: the first one, how many
+    __device__ __forceinline__ P2PLane(int nt, int T, int tid) {
+        const int r = nt & 31;
+        left = r;
+        first = nt - r;
+        target = tid;
+        slice = 0;
+        slices = 1;
+        rest = 0;
+        active = tid < nt;
+        if (r > 0) {
+            const int s = (T - first) / r;
+            rest = s * r;
+            if (tid >= first) {
+                slices = s;
+                slice = (tid - first) / r;
+                target = first + (tid - first) - slice * r;
+                active = slice < s;
+            }
+        }
+    }
+    // The slices' sums added in slice order (block-wide call; `buf` holds one
+    // double4 per thread). Returns whether this thread owns a target's sum.
+    __device__ __forceinline__ bool combine(double4 &v, double4 *buf) const {
+        if (rest <= left) return active;  // one slice each (uniform over the block)
+        const int k = (int)threadIdx.x - first;
+        __syncthreads();
+        if (k >= 0 && active) buf[k] = v;
+        __syncthreads();
+        if (k < 0) return active;
+        if (k >= left) return false;
+        for (int j = k + left; j < rest; j += left) {
+            const double4 o = buf[j];
+            v.x += o.x;
+            v.y += o.y;
+            v.z += o.z;
+            v.w += o.w;
+        }
+        return true;
+    }
+};
 
 // Block b of a batched launch belongs to system s with off[s] <= b < off[s+1].
 __device__ __forceinline__ int batch_sys_of(const int32_t *__restrict__ off, int nsys, int64_t b) {

@@ -462,6 +462,22 @@ cudaError_t scan_exclusive(Plan &P, const int32_t *in, int32_t *out, int64_t n) 
 // it with int32. Lowered only by fmm_set_list_capacity (tests).
 std::atomic<long long> g_list_capacity{0x7fffffffLL};
 
+// Sources per near-field unit (about). A leaf's whole list up to
+// kP2PSegSources where the leaves' tiles alone give every SM kP2PUnitsPerSM
+// units; fewer leaves are cut into as many segments as make up that number,
+// down to kP2PSegMin sources (below, a unit's set-up outweighs its pairs).
+// 64 leaves of 78 points, every list the whole set: 225 us as 64 units, 43 us
+// as 1280. From 10 units per SM on, whole lists cost no more (the units go
+// heaviest first).
+static long long p2p_segment(const Plan &P) {
+    const int64_t nl = P.nleaf, want = (int64_t)kP2PUnitsPerSM * sm_count();
+    const int64_t units = nl * std::max<int64_t>(1, (P.n / nl + P.p2p_tile - 1) / P.p2p_tile);
+    if (units >= want) return kP2PSegSources;
+    const int64_t k = (want + units - 1) / units;
+    const double mean = (double)P.nstrong[P.B] * (double)P.n / ((double)nl * (double)nl);  // sources of a mean list
+    return std::min<long long>(kP2PSegSources, std::max<long long>(kP2PSegMin, (long long)(mean / (double)k) + 1));
+}
+
 cudaError_t lists_build(Plan &P) {
     cudaStream_t st = P.stream;
     // every box's centre split hi + lo in float and its radius, for the
@@ -549,6 +565,7 @@ cudaError_t lists_build(Plan &P) {
     const int64_t nl = (int64_t)1 << P.B;
     P.p2p_tile = (P.prec == FMM_PREC_MIXED && P.n <= (int64_t)kP2PTileSmall * nl) ? kP2PTileSmall : kP2PTile;
     const int tile = P.p2p_tile;
+    const long long smax = p2p_segment(P);
     P.p2p_work_dev = (unsigned long long *)palloc(P, 24);  // pairs, units, partial slots
     long long *nsrc = (long long *)dalloc(P, (size_t)nl * 8);
     int32_t *upl = (int32_t *)dalloc(P, (size_t)nl * 4);
@@ -558,7 +575,7 @@ cudaError_t lists_build(Plan &P) {
     if (!P.p2p_work_dev || !nsrc || !upl || !ppl || !uoff || !P.p2p_poff) return cudaErrorMemoryAllocation;
     cudaMemsetAsync(P.p2p_work_dev, 0, 24, st);
     const unsigned wgrid = (unsigned)std::min<int64_t>((nl * 32 + 255) / 256, (int64_t)sm_count() * 32);
-    FMM_LAUNCH(k_p2p_work, wgrid, 256, 0, st, P.B, tile, (long long)kP2PSegSources,
+    FMM_LAUNCH(k_p2p_work, wgrid, 256, 0, st, P.B, tile, smax,
                P.sptr[P.B], P.ssrc[P.B], P.count, P.p2p_work_dev, nsrc, upl, ppl);
     e = scan_exclusive(P, upl, uoff, nl);
     if (e == cudaSuccess) e = scan_exclusive(P, ppl, P.p2p_poff, nl);
@@ -588,7 +605,7 @@ cudaError_t lists_build(Plan &P) {
         return cudaErrorMemoryAllocation;
     P.p2p_nunits_dev = uoff + nl;
     P.p2p_nunits = nunits;
-    FMM_LAUNCH(k_units_gen, wgrid, 256, 0, st, P.B, tile, (long long)kP2PSegSources,
+    FMM_LAUNCH(k_units_gen, wgrid, 256, 0, st, P.B, tile, smax,
                P.count, nsrc, P.sptr[P.B], P.ssrc[P.B], uoff, P.p2p_poff, units, upart, bucket);
     FMM_LAUNCH(k_units_hist, (unsigned)nblk, kUnitBlock, 0, st, P.p2p_nunits_dev, bucket, nblk, bh);
     e = scan_exclusive(P, bh, boff, (int64_t)256 * nblk);

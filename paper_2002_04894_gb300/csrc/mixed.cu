@@ -407,7 +407,8 @@ __device__ __forceinline__ void block_excl_scan(int *v, int len, int *wsum) {
 // Near field in float. One CTA per work unit (a tile of up to T = 128 or 64
 // targets of one leaf, by the plan's mean leaf size; heaviest units first),
 // one target point per thread, two sources per step in packed float2
-// arithmetic (FFMA2/FADD2/FMUL2). For
+// arithmetic (FFMA2/FADD2/FMUL2); the lanes left over by the tile's last
+// targets take slices of the sources (P2PLane). For
 // every source leaf the offset between the two leaf centres is formed once,
 // error-free (float TwoSum on the centres' hi/lo parts), together with a
 // near/far flag: far when the gap g between the two cells is at least
@@ -452,10 +453,13 @@ __device__ __forceinline__ void p2p_f32_body(int B, int64_t n, const float *__re
     const int e0 = unit.z, e1 = unit.w;  // this unit's segment of the strong list
     const float4 tc_h = geo[3 * t], tc_l = geo[3 * t + 1], tc_e = geo[3 * t + 2];
     const int tid = threadIdx.x;
-    const int i = unit.y + tid;
-    const bool active = i < nt;
+    __shared__ int ntile;  // the tile's targets, for the lanes' roles after the loop (kept in registers they cost occupancy)
+    if (tid == 0) ntile = min(T, nt - unit.y);
+    const P2PLane L(min(T, nt - unit.y), T, tid);
+    const int i = unit.y + L.target, S = L.slices, slice = L.slice;
+    const bool active = L.active;
     // a warp with no target of the unit stages sources and keeps the barriers
-    // but skips the products (the warps past a small leaf's last target)
+    // but skips the products
     const bool busy = __any_sync(0xffffffffu, active);  // warp-uniform
     float xh = 0.f, yh = 0.f, zh = 0.f, xl = 0.f, yl = 0.f, zl = 0.f;
     if (active) {
@@ -471,6 +475,20 @@ __device__ __forceinline__ void p2p_f32_body(int B, int64_t n, const float *__re
     // runs of 64 staged sources (m of them from pair slot 0) against this
     // thread's target, each run compensated into the sums
     auto far_runs = [&](int m) {
+        if (S > 1) {  // warp-uniform: every S-th pair, kRun / 2 of them to a run
+            const int np = (m + 1) >> 1;
+            for (int j0 = 0; j0 < (busy ? np : 0); j0 += S * (kRun / 2)) {
+                const int end = min(np, j0 + S * (kRun / 2));
+                float2 a[4];
+#pragma unroll
+                for (int c = 0; c < 4; c++) a[c] = make_float2(0.f, 0.f);
+#pragma unroll 4
+                for (int pp = j0 + slice; pp < end; pp += S) far_pair2(X, Y, Z, sA[pp], sB[pp], a);
+#pragma unroll
+                for (int c = 0; c < 4; c++) kahan(sum[c], comp[c], a[c].x + a[c].y);
+            }
+            return;
+        }
         for (int j0 = 0; j0 < (busy ? m : 0); j0 += kRun) {
             const int npair = (min(kRun, m - j0) + 1) >> 1;
             const int p0 = j0 >> 1;
@@ -575,6 +593,21 @@ __device__ __forceinline__ void p2p_f32_body(int B, int64_t n, const float *__re
             }
             __syncthreads();
             const int m = min(kNearCap, nnear - base);
+            if (S > 1) {
+                const int np = (m + 1) >> 1;
+                for (int j0 = 0; j0 < (busy ? np : 0); j0 += S * (kRun / 2)) {
+                    const int end = min(np, j0 + S * (kRun / 2));
+                    float2 a[4];
+#pragma unroll
+                    for (int c = 0; c < 4; c++) a[c] = make_float2(0.f, 0.f);
+#pragma unroll 2
+                    for (int pp = j0 + slice; pp < end; pp += S)
+                        near_pair2(X, Y, Z, XL, YL, ZL, sA[pp], sB[pp], sC[pp], sD[pp], a);
+#pragma unroll
+                    for (int c = 0; c < 4; c++) kahan(sum[c], comp[c], a[c].x + a[c].y);
+                }
+                continue;
+            }
             for (int j0 = 0; j0 < (busy ? m : 0); j0 += kRun) {
                 const int npair = (min(kRun, m - j0) + 1) >> 1;
                 const int p0 = j0 >> 1;
@@ -595,30 +628,35 @@ __device__ __forceinline__ void p2p_f32_body(int B, int64_t n, const float *__re
             }
         }
     }
-    if (active && part >= 0) {  // one segment of a split leaf: its partial sums
-        partial[part + i] = make_double4((double)sum[0] - (double)comp[0], (double)sum[1] - (double)comp[1],
-                                         (double)sum[2] - (double)comp[2], (double)sum[3] - (double)comp[3]);
-    } else if (active) {
-        const int64_t a = bt + i;
+    double4 v = make_double4((double)sum[0] - (double)comp[0], (double)sum[1] - (double)comp[1],
+                             (double)sum[2] - (double)comp[2], (double)sum[3] - (double)comp[3]);
+    __syncthreads();
+    const P2PLane M(*(volatile int *)&ntile, T, tid);
+    const bool owner = M.combine(v, (double4 *)sA);
+    const int io = unit.y + M.target;
+    if (owner && part >= 0) {  // one segment of a split leaf: its partial sums
+        partial[part + io] = v;
+    } else if (owner) {
+        const int64_t a = bt + io;
         const int64_t o = perm[a];
-        pot[o] = (OutT)((double)far_phi[a] + ((double)sum[0] - (double)comp[0]));
+        pot[o] = (OutT)((double)far_phi[a] + v.x);
         if (field) {
-            field[3 * o] = (OutT)((double)far_E[a] + ((double)sum[1] - (double)comp[1]));
-            field[3 * o + 1] = (OutT)((double)far_E[n + a] + ((double)sum[2] - (double)comp[2]));
-            field[3 * o + 2] = (OutT)((double)far_E[2 * n + a] + ((double)sum[3] - (double)comp[3]));
+            field[3 * o] = (OutT)((double)far_E[a] + v.y);
+            field[3 * o + 1] = (OutT)((double)far_E[n + a] + v.z);
+            field[3 * o + 2] = (OutT)((double)far_E[2 * n + a] + v.w);
         }
     }
 }
 
-// resident blocks asked of the register allocator (0: no constraint). The
-// batched kernel holds the system's pointers in registers; unconstrained it
-// takes 126 registers. At 64 registers for 128-target tiles (8 blocks) and 80
-// for 64-target tiles (12 blocks) the 512-system batch ran in 319.0 ms, against
-// 324.8 ms at 80 registers for both (328 ms at 72). The single-plan kernel runs
-// best unconstrained (64 registers for 128-target tiles, 64 for 64: with 72 the
-// 8M-point near field took 55.4 instead of 53.3 ms).
+// Resident blocks asked of the register allocator (0: no constraint). The
+// batched kernel holds the system's pointers in registers; at 64 registers for
+// 128-target tiles (8 blocks) and 80 for 64-target tiles (12 blocks) the
+// 512-system batch ran in 319.0 ms, against 324.8 ms at 80 registers for both
+// (328 ms at 72). The single-plan kernel takes 8 blocks for 128-target tiles
+// (16.4 ms on 2M points; 16.9 with 7) and is left unconstrained for 64-target
+// tiles (61.2 ms on 8M points at 96 registers; 61.7 with 14 blocks).
 template <int T>
-constexpr int p2p_min_blocks(bool batched) { return batched ? (T == kP2PTile ? 8 : 12) : 0; }
+constexpr int p2p_min_blocks(bool batched) { return T == kP2PTile ? 8 : batched ? 12 : 0; }
 
 template <typename OutT, int T>
 __global__ void __launch_bounds__(T, p2p_min_blocks<T>(false))

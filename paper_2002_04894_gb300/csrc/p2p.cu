@@ -44,52 +44,51 @@ k_p2p_f64(int B, int64_t npts, const double *__restrict__ x, const double *__res
     const int t = unit.x;
     const int bt = begin[off + t], nt = count[off + t];
     const int e0 = unit.z, e1 = unit.w;  // this unit's segment of the strong list
-    {
-        const int tb = unit.y;
-        const int i = tb + threadIdx.x;
-        const bool active = i < nt;
-        // a warp with no target of the unit stages sources and keeps the
-        // barriers, but skips the products (small leaves: the warps past the
-        // leaf's last target cost no arithmetic)
-        const bool busy = __any_sync(0xffffffffu, active);  // warp-uniform
-        const double xi = active ? x[bt + i] : 0.0;
-        const double yi = active ? y[bt + i] : 0.0;
-        const double zi = active ? z[bt + i] : 0.0;
-        double phi = 0.0, ex = 0.0, ey = 0.0, ez = 0.0;
-        for (int e = e0; e < e1; e++) {
-            const int64_t gs = off + ssrc[e];
-            const int bs = begin[gs], ns = count[gs];
-            for (int sb = 0; sb < ns; sb += kP2PThreads) {
-                const int j = sb + threadIdx.x;
-                tile[threadIdx.x] = j < ns ? Src{x[bs + j], y[bs + j], z[bs + j], q[bs + j]} : Src{0.0, 0.0, 0.0, 0.0};
-                __syncthreads();
-                const int mcount = min(kP2PThreads, ns - sb);
-                for (int jj = 0; jj < (busy ? mcount : 0); jj++) {
-                    const Src s = tile[jj];
-                    const double dx = xi - s.x, dy = yi - s.y, dz = zi - s.z;
-                    const double r2 = dx * dx + dy * dy + dz * dz;
-                    const double rinv = r2 > 0.0 ? rsqrt(r2) : 0.0;
-                    const double qr = s.q * rinv;
-                    const double qr3 = qr * rinv * rinv;
-                    phi += qr;
-                    ex += qr3 * dx;
-                    ey += qr3 * dy;
-                    ez += qr3 * dz;
-                }
-                __syncthreads();
+    const P2PLane L(min(kP2PThreads, nt - unit.y), kP2PThreads, threadIdx.x);
+    const int i = unit.y + L.target;
+    const bool active = L.active;
+    // a warp with no target of the unit stages sources and keeps the
+    // barriers, but skips the products
+    const bool busy = __any_sync(0xffffffffu, active);  // warp-uniform
+    const double xi = active ? x[bt + i] : 0.0;
+    const double yi = active ? y[bt + i] : 0.0;
+    const double zi = active ? z[bt + i] : 0.0;
+    double phi = 0.0, ex = 0.0, ey = 0.0, ez = 0.0;
+    for (int e = e0; e < e1; e++) {
+        const int64_t gs = off + ssrc[e];
+        const int bs = begin[gs], ns = count[gs];
+        for (int sb = 0; sb < ns; sb += kP2PThreads) {
+            const int j = sb + threadIdx.x;
+            tile[threadIdx.x] = j < ns ? Src{x[bs + j], y[bs + j], z[bs + j], q[bs + j]} : Src{0.0, 0.0, 0.0, 0.0};
+            __syncthreads();
+            const int mcount = min(kP2PThreads, ns - sb);
+            for (int jj = L.slice; jj < (busy ? mcount : 0); jj += L.slices) {
+                const Src s = tile[jj];
+                const double dx = xi - s.x, dy = yi - s.y, dz = zi - s.z;
+                const double r2 = dx * dx + dy * dy + dz * dz;
+                const double rinv = r2 > 0.0 ? rsqrt(r2) : 0.0;
+                const double qr = s.q * rinv;
+                const double qr3 = qr * rinv * rinv;
+                phi += qr;
+                ex += qr3 * dx;
+                ey += qr3 * dy;
+                ez += qr3 * dz;
             }
+            __syncthreads();
         }
-        if (active && part >= 0) {  // one segment of a split leaf: its partial sums
-            partial[part + i] = make_double4(phi, ex, ey, ez);
-        } else if (active) {
-            const int64_t a = bt + i;
-            const int64_t o = perm[a];
-            pot[o] = (OutT)(far_phi[a] + phi);
-            if (field) {
-                field[3 * o] = (OutT)(far_E[a] + ex);
-                field[3 * o + 1] = (OutT)(far_E[npts + a] + ey);
-                field[3 * o + 2] = (OutT)(far_E[2 * npts + a] + ez);
-            }
+    }
+    double4 v = make_double4(phi, ex, ey, ez);
+    const bool owner = L.combine(v, (double4 *)tile);
+    if (owner && part >= 0) {  // one segment of a split leaf: its partial sums
+        partial[part + i] = v;
+    } else if (owner) {
+        const int64_t a = bt + i;
+        const int64_t o = perm[a];
+        pot[o] = (OutT)(far_phi[a] + v.x);
+        if (field) {
+            field[3 * o] = (OutT)(far_E[a] + v.y);
+            field[3 * o + 1] = (OutT)(far_E[npts + a] + v.z);
+            field[3 * o + 2] = (OutT)(far_E[2 * npts + a] + v.w);
         }
     }
 }
