@@ -925,7 +925,7 @@ k_b_m2m_up(const BatchSys *__restrict__ S, const int32_t *__restrict__ off, int 
 }
 
 // The whole downward pass (binary levels) in one launch: warps take boxes in
-// chunks of kL2LChunk from one counter in heap order (level by level), so a
+// chunks (of kL2LChunk; see l2l_down) from one counter in heap order (level by level), so a
 // box's parent was taken earlier by a running warp; a box whose parent holds
 // a local expansion (parent level >= lw) waits for the parent's flag, then
 // adds the parent's L2L to its own expansion and raises its flag. Each wait
@@ -973,18 +973,18 @@ __device__ __forceinline__ void l2l_chunk(int lw, int p, const TrIn &a, const do
 template <bool DFT>
 __global__ void __launch_bounds__(kWarpChildMax * 32)
 k_l2l_down(int B, int lw, int p, TrIn a, double2 *L, int *done, unsigned long long *next, int *err,
-           long long wait_limit, long long withhold) {
+           int chunk, long long wait_limit, long long withhold) {
     extern __shared__ double2 sw[];
     const void *tab = stage_tables<DFT>(p, a, sw);
     const int lane = threadIdx.x & 31;
     const int64_t nbox = ((int64_t)2 << B) - 1;
     for (;;) {
         unsigned long long c0 = 0;
-        if (lane == 0) c0 = atomicAdd(next, (unsigned long long)kL2LChunk);
+        if (lane == 0) c0 = atomicAdd(next, (unsigned long long)chunk);
         c0 = __shfl_sync(0xffffffffu, c0, 0);
         if ((int64_t)c0 + 1 >= nbox) break;
         l2l_chunk<DFT>(lw, p, a, nullptr, L, tab, sw, done, err, (int64_t)c0 + 1,
-                       std::min<int64_t>((int64_t)c0 + 1 + kL2LChunk, nbox), wait_limit, withhold);
+                       std::min<int64_t>((int64_t)c0 + 1 + chunk, nbox), wait_limit, withhold);
     }
 }
 
@@ -1231,14 +1231,20 @@ void l2l_down(Plan &P, int lw) {
     cudaMemsetAsync(P.l2l_done, 0, (size_t)P.nbox * 4, P.stream);
     cudaMemsetAsync(P.l2l_next, 0, 8, P.stream);
     const int w = kWarpChildMax;
-    const int64_t items = (P.nbox + kL2LChunk - 1) / kL2LChunk;
+    // A level is done when its last chunk is, box after box in one warp: with
+    // chunks of 8 every level of a small tree took 8 boxes' time (8 levels,
+    // 511 boxes, p = 12: 0.44 ms). Chunks grow only once the boxes outnumber
+    // the resident warps (about 16 per SM) twice.
+    const int chunk =
+        (int)std::max<int64_t>(1, std::min<int64_t>(kL2LChunk, P.nbox / (2 * 16 * (int64_t)sm_count())));
+    const int64_t items = (P.nbox + chunk - 1) / chunk;
     const unsigned grid = (unsigned)std::min<int64_t>((items + w - 1) / w, (int64_t)sm_count() * 8);
     if (df_translations(P))
         FMM_LAUNCH(k_l2l_down<true>, grid, 32 * w, warp_child_smem(P.p, w), P.stream, P.B, lw, P.p, tr_in(P), P.L,
-                   P.l2l_done, P.l2l_next, P.d_err, g_wait_limit.load(), g_withhold.load());
+                   P.l2l_done, P.l2l_next, P.d_err, chunk, g_wait_limit.load(), g_withhold.load());
     else
         FMM_LAUNCH(k_l2l_down<false>, grid, 32 * w, warp_child_smem(P.p, w), P.stream, P.B, lw, P.p, tr_in(P), P.L,
-                   P.l2l_done, P.l2l_next, P.d_err, g_wait_limit.load(), g_withhold.load());
+                   P.l2l_done, P.l2l_next, P.d_err, chunk, g_wait_limit.load(), g_withhold.load());
 }
 
 // FP64 M2L over all levels in one launch; accumulates into L (zeroed first)
