@@ -353,8 +353,10 @@ int fmm_plan(const void *points, int64_t n, int dtype, const fmm_opts *opts,
     if (P.prec == FMM_PREC_MIXED) {
         e = fmm::mixed_setup(P);
         if (e == cudaSuccess) e = fmm::m2l_f32_setup(P);
-        if (e != cudaSuccess) return fail(cuda_status(e));
+    } else {
+        e = fmm::tf_setup(P);
     }
+    if (e != cudaSuccess) return fail(cuda_status(e));
     P.q = (double *)fmm::palloc(P, n * 8);
     P.far_phi = (double *)fmm::palloc(P, n * 8);
     P.far_E = (double *)fmm::palloc(P, n * 24);

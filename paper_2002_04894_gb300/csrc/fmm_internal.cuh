@@ -232,6 +232,11 @@ struct Plan {
     int tc_ctas = 0;
     float2 *Mf = nullptr;
     double2 *Lh = nullptr;  // r^k-scaled locals accumulated by the float M2L
+    // FP64 form's near field: positions on the grid and charges in three
+    // floats, the pair thresholds (positions' own; with the charges'), the
+    // largest charge's exponent
+    float *tf_pos = nullptr, *tf_q = nullptr, *tf_thr0 = nullptr, *tf_thr = nullptr;
+    int *tf_emax = nullptr;
     // evaluation scratch
     double *q = nullptr;                 // charges in leaf order
     double2 *M = nullptr, *L = nullptr;  // nbox x nc
@@ -412,6 +417,8 @@ cudaError_t m2l_tc_setup(Plan &P);
 cudaError_t m2l_tc_launch(Plan &P);
 cudaError_t m2l_f32_setup(Plan &P);
 cudaError_t m2l_f32_all(Plan &P);
+cudaError_t tf_setup(Plan &P);
+cudaError_t tf_p2p(Plan &P, void *pot, void *field, int dtype);
 cudaError_t mixed_setup(Plan &P);
 cudaError_t mixed_p2m(Plan &P, const void *charges, int dtype);
 cudaError_t mixed_l2p(Plan &P);

@@ -1,14 +1,9 @@
-// Near field (P2P, Algorithm 4) and the exact sum of Eq. 2.1.
-//
-// P2P: for every target leaf, the direct interaction with the points of all
-// strongly connected leaves (itself included), pairs at zero distance
-// skipped. One CTA per work unit (a tile of a target leaf's points against a
-// segment of its strong list), one target point per thread; source leaves
-// are staged through shared memory in tiles of (x, y, z, q). The kernel adds
-// the far field left by L2P and writes phi and E straight to the caller's
-// arrays in input order (the un-permute step); a leaf whose strong list was
-// cut into segments leaves per-segment partial sums instead, which the
-// combine pass adds in segment order.
+// The exact sum of Eq. 2.1 at selected targets, and the end of the near field
+// (P2P, Algorithm 4): its launch by precision form (p2p_tf.cu, mixed.cu; one
+// block per work unit, a tile of a target leaf's points against a segment of
+// its strong list, the far field added and the results written in input
+// order) and the pass that adds the partial sums of leaves whose strong list
+// was cut into segments, in segment order.
 //
 // Direct: one CTA per target, threads stride over all sources with
 // Neumaier-compensated partial sums, then a block reduction.
@@ -20,78 +15,6 @@
 namespace fmm {
 
 namespace {
-
-constexpr int kP2PThreads = 128;
-
-template <typename OutT>
-__global__ void __launch_bounds__(kP2PThreads)
-k_p2p_f64(int B, int64_t npts, const double *__restrict__ x, const double *__restrict__ y,
-          const double *__restrict__ z, const double *__restrict__ q,
-          const int32_t *__restrict__ begin, const int32_t *__restrict__ count,
-          const int32_t *__restrict__ ssrc, const int4 *__restrict__ units, const int32_t *__restrict__ upart,
-          const int32_t *__restrict__ nunits, const int32_t *__restrict__ perm,
-          const double *__restrict__ far_phi, const double *__restrict__ far_E, double4 *__restrict__ partial,
-          OutT *__restrict__ pot, OutT *__restrict__ field) {
-    struct alignas(16) Src {
-        double x, y, z, q;
-    };
-    __shared__ Src tile[kP2PThreads];
-    const int64_t off = ((int64_t)1 << B) - 1;
-    static_assert(kP2PThreads == kP2PTile, "one target per thread");
-    if ((int)blockIdx.x >= *nunits) return;  // launched for an upper bound on the units
-    const int4 unit = units[blockIdx.x];
-    const int part = upart[blockIdx.x];
-    const int t = unit.x;
-    const int bt = begin[off + t], nt = count[off + t];
-    const int e0 = unit.z, e1 = unit.w;  // this unit's segment of the strong list
-    const P2PLane L(min(kP2PThreads, nt - unit.y), kP2PThreads, threadIdx.x);
-    const int i = unit.y + L.target;
-    const bool active = L.active;
-    // a warp with no target of the unit stages sources and keeps the
-    // barriers, but skips the products
-    const bool busy = __any_sync(0xffffffffu, active);  // warp-uniform
-    const double xi = active ? x[bt + i] : 0.0;
-    const double yi = active ? y[bt + i] : 0.0;
-    const double zi = active ? z[bt + i] : 0.0;
-    double phi = 0.0, ex = 0.0, ey = 0.0, ez = 0.0;
-    for (int e = e0; e < e1; e++) {
-        const int64_t gs = off + ssrc[e];
-        const int bs = begin[gs], ns = count[gs];
-        for (int sb = 0; sb < ns; sb += kP2PThreads) {
-            const int j = sb + threadIdx.x;
-            tile[threadIdx.x] = j < ns ? Src{x[bs + j], y[bs + j], z[bs + j], q[bs + j]} : Src{0.0, 0.0, 0.0, 0.0};
-            __syncthreads();
-            const int mcount = min(kP2PThreads, ns - sb);
-            for (int jj = L.slice; jj < (busy ? mcount : 0); jj += L.slices) {
-                const Src s = tile[jj];
-                const double dx = xi - s.x, dy = yi - s.y, dz = zi - s.z;
-                const double r2 = dx * dx + dy * dy + dz * dz;
-                const double rinv = r2 > 0.0 ? rsqrt(r2) : 0.0;
-                const double qr = s.q * rinv;
-                const double qr3 = qr * rinv * rinv;
-                phi += qr;
-                ex += qr3 * dx;
-                ey += qr3 * dy;
-                ez += qr3 * dz;
-            }
-            __syncthreads();
-        }
-    }
-    double4 v = make_double4(phi, ex, ey, ez);
-    const bool owner = L.combine(v, (double4 *)tile);
-    if (owner && part >= 0) {  // one segment of a split leaf: its partial sums
-        partial[part + i] = v;
-    } else if (owner) {
-        const int64_t a = bt + i;
-        const int64_t o = perm[a];
-        pot[o] = (OutT)(far_phi[a] + v.x);
-        if (field) {
-            field[3 * o] = (OutT)(far_E[a] + v.y);
-            field[3 * o + 1] = (OutT)(far_E[npts + a] + v.z);
-            field[3 * o + 2] = (OutT)(far_E[2 * npts + a] + v.w);
-        }
-    }
-}
 
 __device__ __forceinline__ void neumaier(double &s, double &c, double v) {
     const double t = s + v;
@@ -216,22 +139,14 @@ k_b_p2p_combine(const BatchSys *__restrict__ S, const int32_t *__restrict__ off,
 }  // namespace
 
 cudaError_t eval_p2p(Plan &P, void *pot, void *field, int dtype) {
-    const unsigned grid = (unsigned)P.p2p_nunits;
     stage_mark(P, FMM_STAGE_P2P, 0);
     if (P.prec == FMM_PREC_MIXED) {
         cudaError_t e = mixed_p2p(P, pot, field, dtype);
         stage_mark(P, FMM_STAGE_P2P, 1);
         return e;
     }
-    if (dtype == FMM_F64)
-        FMM_LAUNCH(k_p2p_f64<double>, grid, kP2PThreads, 0, P.stream, P.B, P.n, P.x, P.y, P.z, P.q, P.begin,
-                   P.count, P.ssrc[P.B], P.p2p_units, P.p2p_upart, P.p2p_nunits_dev, P.perm, P.far_phi, P.far_E,
-                   P.p2p_partial, (double *)pot, (double *)field);
-    else
-        FMM_LAUNCH(k_p2p_f64<float>, grid, kP2PThreads, 0, P.stream, P.B, P.n, P.x, P.y, P.z, P.q, P.begin,
-                   P.count, P.ssrc[P.B], P.p2p_units, P.p2p_upart, P.p2p_nunits_dev, P.perm, P.far_phi, P.far_E,
-                   P.p2p_partial, (float *)pot, (float *)field);
-    cudaError_t e = p2p_combine(P, pot, field, dtype);
+    cudaError_t e = tf_p2p(P, pot, field, dtype);
+    if (e == cudaSuccess) e = p2p_combine(P, pot, field, dtype);
     stage_mark(P, FMM_STAGE_P2P, 1);
     return e;
 }

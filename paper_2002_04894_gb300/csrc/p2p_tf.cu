@@ -1,0 +1,291 @@
+// Near field of the FP64 form (P2P, Algorithm 4) in three-float arithmetic.
+//
+// What bounds it: the FP32 pipe (84% busy). A pair takes ~360 packed
+// operations (trifloat.cuh) where FP64 arithmetic takes 19 FP64 instructions at
+// less than two per clock and SM, ~1,400 FP32 operations' time, and its terms
+// are more accurate than those of plain double arithmetic. Sums run in
+// TwoSum-compensated three-float accumulators. 200k Plummer points, 11 levels,
+// 1.16e10 pairs: FP64 arithmetic 412.6 ms (its pipe saturated), this 124.5;
+// 20k uniform points, 8 levels: 3.29 -> 1.05 ms. Registers: 4 blocks of 128
+// threads per SM (128 registers; 5 blocks 127.9 ms, 6 132.7). With block-wide
+// staging and its barriers: 152.9 ms.
+//
+// Positions are taken relative to the root cell's centre on a common grid of
+// 2^-72 of its extent (rounded up to a power of two): three floats of 24 bits
+// each, whose differences are exact part by part. A double that does not fit
+// the grid (a coordinate within 2^-19 of the extent of the centre has finer
+// bits) is rounded to it and marked; a pair goes through FP64 arithmetic on the
+// original doubles instead when its distance is below 2^-19 of the extent
+// with a marked point, below 2^-23 otherwise (that includes r = 0), or when
+// the charge is not finite or below 2^-60 of the largest.
+
+#include <algorithm>
+
+#include "fmm_internal.cuh"
+#include "trifloat.cuh"
+
+namespace fmm {
+
+namespace {
+
+constexpr float kThrExact = 0x1p-46f, kThrRounded = 0x1p-38f;  // on r^2 over the squared extent
+
+// exponent k of the grid's extent: 2^k > the root cell's longest side (a side
+// outside the double range's middle: all pairs are left to FP64)
+__device__ __forceinline__ bool grid_exponent(const double *__restrict__ lo, const double *__restrict__ hi, int &k) {
+    const double w = fmax(fmax(hi[0] - lo[0], hi[1] - lo[1]), hi[2] - lo[2]);
+    const int e = w > 0.0 ? ilogb(w) + 1 : 0;
+    const bool ok = w < 0x1p1000 && e > -1000;
+    k = ok ? e : 0;
+    return ok;
+}
+
+// coordinate x (relative to centre c) in three floats; false if rounded
+__device__ __forceinline__ bool grid_split(double x, double c, double inv, float (&f)[3]) {
+    const double u = __dsub_rn(x, c), bb = __dsub_rn(u, x);
+    const double e = __dadd_rn(__dsub_rn(x, __dsub_rn(u, bb)), __dsub_rn(-c, bb));  // x - c = u + e
+    const double us = u * inv, es = e * inv;
+    constexpr double M1 = 0x1.8p28, M2 = 0x1.8p4, M3 = 0x1.8p-20;  // grids 2^-24, 2^-48, 2^-72
+    const double a = __dsub_rn(__dadd_rn(us, M1), M1), r = __dsub_rn(us, a);
+    const double v = __dadd_rn(r, es), vb = __dsub_rn(v, r);
+    const double ve = __dadd_rn(__dsub_rn(r, __dsub_rn(v, vb)), __dsub_rn(es, vb));
+    const double b = __dsub_rn(__dadd_rn(v, M2), M2), s = __dsub_rn(v, b);
+    const double d = __dsub_rn(__dadd_rn(s, M3), M3);
+    f[0] = (float)a, f[1] = (float)b, f[2] = (float)d;
+    return d == s && ve == 0.0;
+}
+
+// plan time: positions on the grid (component-major: [part][axis][n]) and the thresholds they give
+__global__ void k_tf_points(int64_t n, const double *__restrict__ x, const double *__restrict__ y,
+                            const double *__restrict__ z, const double *__restrict__ lo,
+                            const double *__restrict__ hi, float *__restrict__ pos, float *__restrict__ thr) {
+    int k;
+    const bool ok = grid_exponent(lo, hi, k);
+    const double inv = scalbn(1.0, -k);
+    const double *src[3] = {x, y, z};
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        bool exact = true;
+#pragma unroll
+        for (int a = 0; a < 3; a++) {
+            float f[3] = {0.f, 0.f, 0.f};
+            if (ok) exact &= grid_split(src[a][i], 0.5 * lo[a] + 0.5 * hi[a], inv, f);
+#pragma unroll
+            for (int c = 0; c < 3; c++) pos[(3 * c + a) * n + i] = f[c];
+        }
+        thr[i] = !ok ? __int_as_float(0x7f800000) : exact ? kThrExact : kThrRounded;
+    }
+}
+
+// the largest finite charge's exponent (bits of |q| >> 52)
+__global__ void __launch_bounds__(256)
+k_tf_qmax(int64_t n, const double *__restrict__ q, int *__restrict__ emax) {
+    int m = 0;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const int e = (int)((__double_as_longlong(q[i]) >> 52) & 0x7ff);
+        if (e < 0x7ff) m = max(m, e);
+    }
+    m = __reduce_max_sync(0xffffffffu, m);
+    if ((threadIdx.x & 31) == 0 && m > 0) atomicMax(emax, m);
+}
+
+// 2^q_exponent is above every finite charge (all subnormal or zero: 2^-1022)
+__device__ __forceinline__ int q_exponent(int e) { return max(e, 1) - 1022; }
+
+// charges over 2^q_exponent in three floats, and the pair thresholds with the charges' own
+__global__ void __launch_bounds__(256)
+k_tf_charges(int64_t n, const double *__restrict__ q, const int *__restrict__ emax, const float *__restrict__ thr0,
+             float *__restrict__ tq, float *__restrict__ thr) {
+    const int e = q_exponent(*emax);
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const double s = scalbn(q[i], -e), as = fabs(s);
+        const bool ok = as == 0.0 || (as >= 0x1p-60 && as <= 1.0);  // NaN and infinities: no
+        const float a = ok ? (float)s : 0.f;
+        const double r = ok ? s - (double)a : 0.0;
+        const float b = (float)r;
+        tq[i] = a;
+        tq[n + i] = b;
+        tq[2 * n + i] = (float)(r - (double)b);
+        thr[i] = ok ? thr0[i] : __int_as_float(0x7f800000);
+    }
+}
+
+constexpr int kT = kP2PTile;  // threads and targets per unit
+constexpr int kChunk = 64;    // sources staged at a time by a warp
+
+// source j on target i in FP64 on the original positions, pairs at zero distance skipped
+__device__ __noinline__ void pair_f64(const double *__restrict__ x, const double *__restrict__ y,
+                                      const double *__restrict__ z, const double *__restrict__ q, int i, int j,
+                                      double (&s)[4]) {
+    const double dx = x[i] - x[j], dy = y[i] - y[j], dz = z[i] - z[j];
+    const double r2 = dx * dx + dy * dy + dz * dz;
+    const double rinv = r2 > 0.0 ? rsqrt(r2) : 0.0;
+    const double qr = q[j] * rinv, qr3 = qr * rinv * rinv;
+    s[0] += qr;
+    s[1] += qr3 * dx;
+    s[2] += qr3 * dy;
+    s[3] += qr3 * dz;
+}
+
+template <typename OutT>
+__global__ void __launch_bounds__(kT, 4)
+k_p2p_tf(int B, int64_t n, const double *__restrict__ x, const double *__restrict__ y, const double *__restrict__ z,
+         const double *__restrict__ q, const float *__restrict__ pos, const float *__restrict__ tq,
+         const float *__restrict__ thr0, const float *__restrict__ thr, const double *__restrict__ lo,
+         const double *__restrict__ hi, const int *__restrict__ emax, const int32_t *__restrict__ begin,
+         const int32_t *__restrict__ count, const int32_t *__restrict__ ssrc, const int4 *__restrict__ units,
+         const int32_t *__restrict__ upart, const int32_t *__restrict__ nunits, const int32_t *__restrict__ perm,
+         const double *__restrict__ far_phi, const double *__restrict__ far_E, double4 *__restrict__ partial,
+         OutT *__restrict__ pot, OutT *__restrict__ field) {
+    // per warp and source pair: parts a, b, c of (x, y, z, q), the two sources
+    // side by side. Each warp stages its own sources: a chunk is some 20,000
+    // cycles of arithmetic, so four warps loading the same one cost nothing,
+    // and none waits for the others at a barrier.
+    __shared__ float4 sm_all[kT / 32][6][kChunk / 2];
+    __shared__ float2 sthr_all[kT / 32][kChunk / 2];
+    __shared__ double4 red[kT];
+    if ((int)blockIdx.x >= *nunits) return;  // launched for an upper bound on the units
+    const int64_t off = ((int64_t)1 << B) - 1;
+    const int4 unit = units[blockIdx.x];
+    const int part = upart[blockIdx.x];
+    const int t = unit.x, tid = threadIdx.x;
+    const int bt = begin[off + t], nt = count[off + t];
+    const P2PLane L(min(kT, nt - unit.y), kT, tid);
+    const int i = unit.y + L.target, slot = bt + i;
+    const bool busy = __any_sync(0xffffffffu, L.active);  // warp-uniform
+    tf::Tri<float2> X[3];
+    float thr_i = 0.f;
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        float f[3] = {0.f, 0.f, 0.f};
+        if (L.active)
+#pragma unroll
+            for (int c = 0; c < 3; c++) f[c] = pos[(3 * c + a) * n + slot];
+        X[a] = {make_float2(f[0], f[0]), make_float2(f[1], f[1]), make_float2(f[2], f[2])};
+    }
+    if (L.active) thr_i = thr0[slot];
+    const float2 zero = make_float2(0.f, 0.f);
+    tf::Acc<float2> A[4] = {{zero, zero, zero}, {zero, zero, zero}, {zero, zero, zero}, {zero, zero, zero}};
+    double slow[4] = {0.0, 0.0, 0.0, 0.0};
+    float4(*sm)[kChunk / 2] = sm_all[tid >> 5];
+    float2 *sthr = sthr_all[tid >> 5];
+    float *fs = (float *)sm, *ft = (float *)sthr;
+    for (int e = unit.z; e < (busy ? unit.w : 0); e++) {
+        const int64_t gs = off + ssrc[e];
+        const int bs = begin[gs], ns = count[gs];
+        for (int sb = 0; sb < ns; sb += kChunk) {
+            __syncwarp();
+#pragma unroll
+            for (int h = 0; h < kChunk; h += 32) {
+                const int s = h + (tid & 31), j = sb + s;
+                float v[12] = {}, th = 0.f;
+                v[0] = -1.f;  // padding: a zero charge away from every target
+                if (j < ns) {
+#pragma unroll
+                    for (int c = 0; c < 3; c++) {
+#pragma unroll
+                        for (int a = 0; a < 3; a++) v[4 * c + a] = -pos[(3 * c + a) * n + bs + j];
+                        v[4 * c + 3] = tq[c * n + bs + j];
+                    }
+                    th = thr[bs + j];
+                }
+#pragma unroll
+                for (int c = 0; c < 12; c++)
+                    fs[((c >> 1) * (kChunk / 2) + (s >> 1)) * 4 + 2 * (c & 1) + (s & 1)] = v[c];
+                ft[s] = th;
+            }
+            __syncwarp();
+            const int np = (min(kChunk, ns - sb) + 1) >> 1;
+#pragma unroll 1
+            for (int pp = L.slice; pp < np; pp += L.slices) {
+                const float4 a0 = sm[0][pp], a1 = sm[1][pp], b0 = sm[2][pp], b1 = sm[3][pp], c0 = sm[4][pp],
+                             c1 = sm[5][pp];
+                const float2 th = sthr[pp];
+                const tf::Tri<float2> Y[3] = {
+                    {make_float2(a0.x, a0.y), make_float2(b0.x, b0.y), make_float2(c0.x, c0.y)},
+                    {make_float2(a0.z, a0.w), make_float2(b0.z, b0.w), make_float2(c0.z, c0.w)},
+                    {make_float2(a1.x, a1.y), make_float2(b1.x, b1.y), make_float2(c1.x, c1.y)}};
+                const tf::Tri<float2> Q = {make_float2(a1.z, a1.w), make_float2(b1.z, b1.w), make_float2(c1.z, c1.w)};
+                tf::PairTerms<float2> o = tf::pair_terms(X, Y, Q);
+                const bool bx = o.r2.x < fmaxf(th.x, thr_i), by = o.r2.y < fmaxf(th.y, thr_i);
+                if (bx || by) {
+                    const int j0 = sb + 2 * pp;  // the leaf's sources j0 and j0 + 1 (padding past its last one)
+                    if (bx) {
+                        // a target meets itself once: nothing, unless its charge is not finite
+                        if (L.active && (bs + j0 != slot || isinf(th.x))) pair_f64(x, y, z, q, slot, bs + j0, slow);
+                        o.phi.a.x = o.phi.b.x = o.phi.c.x = 0.f;
+#pragma unroll
+                        for (int a = 0; a < 3; a++) o.e[a].a.x = o.e[a].b.x = o.e[a].c.x = 0.f;
+                    }
+                    if (by) {
+                        if (L.active && j0 + 1 < ns && (bs + j0 + 1 != slot || isinf(th.y)))
+                            pair_f64(x, y, z, q, slot, bs + j0 + 1, slow);
+                        o.phi.a.y = o.phi.b.y = o.phi.c.y = 0.f;
+#pragma unroll
+                        for (int a = 0; a < 3; a++) o.e[a].a.y = o.e[a].b.y = o.e[a].c.y = 0.f;
+                    }
+                }
+                A[0].put(o.phi);
+#pragma unroll
+                for (int a = 0; a < 3; a++) A[1 + a].put(o.e[a]);
+            }
+        }
+    }
+    int k;
+    grid_exponent(lo, hi, k);
+    const int eq = q_exponent(*emax);
+    double v[4];
+#pragma unroll
+    for (int c = 0; c < 4; c++)
+        v[c] = scalbn(((double)A[c].a.x + (double)A[c].a.y) +
+                          (((double)A[c].b.x + (double)A[c].b.y) + ((double)A[c].c.x + (double)A[c].c.y)),
+                      c ? eq - 2 * k : eq - k) +
+               slow[c];
+    double4 r = make_double4(v[0], v[1], v[2], v[3]);
+    const bool owner = L.combine(r, red);
+    if (owner && part >= 0) {  // one segment of a split leaf: its partial sums
+        partial[part + i] = r;
+    } else if (owner) {
+        const int64_t o = perm[slot];
+        pot[o] = (OutT)(far_phi[slot] + r.x);
+        if (field) {
+            field[3 * o] = (OutT)(far_E[slot] + r.y);
+            field[3 * o + 1] = (OutT)(far_E[n + slot] + r.z);
+            field[3 * o + 2] = (OutT)(far_E[2 * n + slot] + r.w);
+        }
+    }
+}
+
+unsigned grid_for(int64_t n) { return (unsigned)std::min<int64_t>((n + 255) / 256, (int64_t)sm_count() * 8); }
+
+}  // namespace
+
+cudaError_t tf_setup(Plan &P) {
+    const size_t n = (size_t)P.n;
+    P.tf_pos = (float *)palloc(P, n * 36);
+    P.tf_q = (float *)palloc(P, n * 12);
+    P.tf_thr0 = (float *)palloc(P, n * 4);
+    P.tf_thr = (float *)palloc(P, n * 4);
+    P.tf_emax = (int *)palloc(P, 4);
+    if (!P.tf_pos || !P.tf_q || !P.tf_thr0 || !P.tf_thr || !P.tf_emax) return cudaErrorMemoryAllocation;
+    FMM_LAUNCH(k_tf_points, grid_for(P.n), 256, 0, P.stream, P.n, P.x, P.y, P.z, P.lo, P.hi, P.tf_pos, P.tf_thr0);
+    return cudaGetLastError();
+}
+
+cudaError_t tf_p2p(Plan &P, void *pot, void *field, int dtype) {
+    cudaMemsetAsync(P.tf_emax, 0, 4, P.stream);
+    FMM_LAUNCH(k_tf_qmax, grid_for(P.n), 256, 0, P.stream, P.n, P.q, P.tf_emax);
+    FMM_LAUNCH(k_tf_charges, grid_for(P.n), 256, 0, P.stream, P.n, P.q, P.tf_emax, P.tf_thr0, P.tf_q, P.tf_thr);
+    if (dtype == FMM_F64)
+        FMM_LAUNCH(k_p2p_tf<double>, (unsigned)P.p2p_nunits, kT, 0, P.stream, P.B, P.n, P.x, P.y, P.z, P.q, P.tf_pos,
+                   P.tf_q, P.tf_thr0, P.tf_thr, P.lo, P.hi, P.tf_emax, P.begin, P.count, P.ssrc[P.B], P.p2p_units,
+                   P.p2p_upart, P.p2p_nunits_dev, P.perm, P.far_phi, P.far_E, P.p2p_partial, (double *)pot,
+                   (double *)field);
+    else
+        FMM_LAUNCH(k_p2p_tf<float>, (unsigned)P.p2p_nunits, kT, 0, P.stream, P.B, P.n, P.x, P.y, P.z, P.q, P.tf_pos,
+                   P.tf_q, P.tf_thr0, P.tf_thr, P.lo, P.hi, P.tf_emax, P.begin, P.count, P.ssrc[P.B], P.p2p_units,
+                   P.p2p_upart, P.p2p_nunits_dev, P.perm, P.far_phi, P.far_E, P.p2p_partial, (float *)pot,
+                   (float *)field);
+    return cudaGetLastError();
+}
+
+}  // namespace fmm

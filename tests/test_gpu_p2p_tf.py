@@ -1,0 +1,64 @@
+"""The FP64 form's near field (three-float arithmetic, FP64 for the pairs it
+cannot hold) against the exact sum in extended precision, theta = 0.
+
+Tolerance per target: a pair's terms are accurate to 2^-52 relative (FP64
+pairs: a few ulp, < 2^-50), the sums add less, and the result is rounded once:
+|err| <= 2^-49 sum_j |q_j| / r for the potential, 2^-48 sum_j |q_j| / r^2 for each
+field component."""
+import numpy as np
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+def cloud(kind, n, rng):
+    x = rng.random((n, 3))
+    q = rng.uniform(-1.0, 1.0, n)
+    if kind == "close":          # distances from 1e-1 down to 1e-15 around a few points
+        x = x[rng.integers(0, 5, n)] + 10.0 ** rng.uniform(-15, -1, (n, 1)) * rng.normal(size=(n, 3))
+        x[3] = x[9]
+    elif kind == "centre":       # fine bits: clusters at the root cell's centre and at the origin
+        x = (x - 0.5) * 10.0 ** rng.uniform(-12, 0, (n, 1))
+        x[0], x[1] = (-0.5, -0.5, -0.5), (0.5, 0.5, 0.5)
+    elif kind == "offset":
+        x = x + 1.0e6
+    elif kind == "huge":
+        x = x * 1e120
+    elif kind == "tiny":
+        x, q = x * 1e-120, q * 1.6e-19
+    elif kind == "charges":      # magnitudes from 1 down to 1e-40, zeros
+        q = q * 10.0 ** rng.uniform(-40, 0, n)
+        q[::7] = 0.0
+    elif kind == "plane":
+        x[:, 2] = 0.25
+    elif kind == "line":
+        x[:, 1:] = 0.0
+    return x, q
+
+
+@pytest.mark.parametrize("levels", [0, 3])
+@pytest.mark.parametrize("kind", ["uniform", "close", "centre", "offset", "huge", "tiny", "charges", "plane", "line"])
+def test_matches_extended_precision(gpu_lib, kind, levels):
+    fmm = gpu_lib
+    x, q = cloud(kind, 333, np.random.default_rng(17))
+    plan = fmm.fmm_plan(torch.from_numpy(x).cuda(), levels, 2, 0.0)
+    pot, fld = (t.cpu().numpy() for t in fmm.fmm_eval(plan, torch.from_numpy(q).cuda()))
+    X, Q = x.astype(np.longdouble), q.astype(np.longdouble)
+    d = X[:, None, :] - X[None, :, :]
+    r = np.sqrt((d * d).sum(-1))
+    w = np.divide(np.longdouble(1), r, out=np.zeros_like(r), where=r > 0)
+    phi, mag = (w * Q).sum(1), (w * abs(Q)).sum(1)
+    E, magE = ((w ** 3 * Q)[:, :, None] * d).sum(1), (w ** 2 * abs(Q)).sum(1)
+    assert np.all(abs(pot - phi) <= 2.0 ** -49 * mag)
+    assert np.all(abs(fld - E) <= 2.0 ** -48 * magE[:, None])
+
+
+def test_non_finite_charge_reaches_every_target(gpu_lib):
+    fmm = gpu_lib
+    x, q = cloud("uniform", 100, np.random.default_rng(3))
+    for bad in (np.inf, np.nan):
+        q[41] = bad
+        plan = fmm.fmm_plan(torch.from_numpy(x).cuda(), 2, 2, 0.0)
+        pot = fmm.fmm_eval(plan, torch.from_numpy(q).cuda())[0].cpu().numpy()
+        assert not np.isfinite(pot).any()
