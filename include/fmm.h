@@ -66,7 +66,8 @@ enum fmm_dtype { FMM_F64 = 0, FMM_F32 = 1 };
 
 /*
  * Arithmetic of the evaluation stages.
- *  FMM_PREC_FP64  every stage in double precision (the plain form).
+ *  FMM_PREC_FP64  every stage in double precision or better (the plain form;
+ *                 the near field in sums of three floats, ~72 bits).
  *  FMM_PREC_MIXED box geometry, theta-test, M2M and L2L in double; P2M, M2L,
  *                 L2P and P2P in single precision with leaf-centred
  *                 coordinates and compensated per-target sums.
@@ -200,8 +201,11 @@ void fmm_destroy(fmm_plan_t plan);
  *   points, charges  n x 3 and n values (dtype), host or device.
  *   targets          ntargets int64 indices into [0, n), host or device.
  *   potentials       ntargets outputs (dtype); fields: ntargets x 3 or NULL.
- * Sources are summed in blocks with compensated (Neumaier) partial sums.
- * Allocates device staging only for host arguments (cudaMallocAsync).
+ * The pairs run in three-float arithmetic with compensated sums (relative
+ * errors below those of double arithmetic), pairs it cannot hold in double.
+ * Takes its workspace (up to about 58 MB, and 32 bytes per target and source
+ * segment) from the library's stream-ordered pool and gives it back before it
+ * returns; device staging for host arguments with cudaMallocAsync.
  * Errors: FMM_EINVAL (n < 1, ntargets < 0, NULL pointers), FMM_ECUDA.
  */
 int fmm_direct(const void *points, const void *charges, int64_t n, int dtype,

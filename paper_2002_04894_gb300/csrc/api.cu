@@ -89,18 +89,26 @@ cudaMemPool_t library_pool(int dev) {
     return g_pool[dev];
 }
 
-void *raw_alloc(Plan &P, size_t bytes) {
-    if (P.has_alloc) return P.alloc.alloc(bytes, P.alloc.ctx, (void *)P.stream);
+}  // namespace
+
+void *pool_alloc(size_t bytes, cudaStream_t st) {
     int dev = 0;
     void *p = nullptr;
     cudaMemPool_t pool = cudaGetDevice(&dev) == cudaSuccess ? library_pool(dev) : nullptr;
-    const cudaError_t e = pool ? cudaMallocFromPoolAsync(&p, bytes, pool, P.stream)
-                               : cudaMallocAsync(&p, bytes, P.stream);
+    const cudaError_t e = pool ? cudaMallocFromPoolAsync(&p, bytes, pool, st) : cudaMallocAsync(&p, bytes, st);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return nullptr;
     }
     return p;
+}
+void pool_free(void *p, cudaStream_t st) { cudaFreeAsync(p, st); }
+
+namespace {
+
+void *raw_alloc(Plan &P, size_t bytes) {
+    if (P.has_alloc) return P.alloc.alloc(bytes, P.alloc.ctx, (void *)P.stream);
+    return pool_alloc(bytes, P.stream);
 }
 
 void raw_free(Plan &P, void *ptr, size_t bytes) {

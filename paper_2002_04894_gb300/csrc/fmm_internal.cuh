@@ -417,6 +417,11 @@ cudaError_t m2l_tc_setup(Plan &P);
 cudaError_t m2l_tc_launch(Plan &P);
 cudaError_t m2l_f32_setup(Plan &P);
 cudaError_t m2l_f32_all(Plan &P);
+// stream-ordered workspace from the library's own pool of the current device (null: none to be had)
+void *pool_alloc(size_t bytes, cudaStream_t st);
+void pool_free(void *p, cudaStream_t st);
+cudaError_t direct_tf(const void *pts, const void *q, int64_t n, int dtype, const int64_t *targets, int64_t nt,
+                      void *pot, void *field, cudaStream_t st);
 cudaError_t tf_setup(Plan &P);
 cudaError_t tf_p2p(Plan &P, void *pot, void *field, int dtype);
 cudaError_t mixed_setup(Plan &P);

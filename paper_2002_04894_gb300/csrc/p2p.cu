@@ -5,8 +5,9 @@
 // order) and the pass that adds the partial sums of leaves whose strong list
 // was cut into segments, in segment order.
 //
-// Direct: one CTA per target, threads stride over all sources with
-// Neumaier-compensated partial sums, then a block reduction.
+// Direct: p2p_tf.cu; where its workspace cannot be had, one CTA per target in
+// FP64, threads striding over all sources with Neumaier-compensated partial
+// sums, then a block reduction.
 
 #include <algorithm>
 
@@ -174,6 +175,9 @@ cudaError_t direct_run(const void *points, const void *charges, int64_t n, int d
                        const int64_t *targets, int64_t nt, void *pot, void *field,
                        cudaStream_t s) {
     if (nt == 0) return cudaSuccess;
+    const cudaError_t e = direct_tf(points, charges, n, dtype, targets, nt, pot, field, s);
+    if (e != cudaErrorMemoryAllocation) return e;
+    // no workspace to be had: one block per target in FP64
     if (dtype == FMM_F64)
         FMM_LAUNCH(k_direct<double>, (unsigned)nt, 256, 0, s, (const double *)points, (const double *)charges,
                                                       n, targets, (double *)pot, (double *)field);

@@ -91,21 +91,50 @@ k_tf_qmax(int64_t n, const double *__restrict__ q, int *__restrict__ emax) {
 // 2^q_exponent is above every finite charge (all subnormal or zero: 2^-1022)
 __device__ __forceinline__ int q_exponent(int e) { return max(e, 1) - 1022; }
 
+// a charge over 2^e in three floats; its pairs' threshold
+__device__ __forceinline__ float charge_split(double q, int e, float thr, float (&f)[3]) {
+    const double s = scalbn(q, -e), as = fabs(s);
+    const bool ok = as == 0.0 || (as >= 0x1p-60 && as <= 1.0);  // NaN and infinities: no
+    f[0] = ok ? (float)s : 0.f;
+    const double r = ok ? s - (double)f[0] : 0.0;
+    f[1] = (float)r;
+    f[2] = (float)(r - (double)f[1]);
+    return ok ? thr : __int_as_float(0x7f800000);
+}
+
+__device__ __forceinline__ void clear_x(tf::PairTerms<float2> &o) {
+    o.phi.a.x = o.phi.b.x = o.phi.c.x = 0.f;
+#pragma unroll
+    for (int a = 0; a < 3; a++) o.e[a].a.x = o.e[a].b.x = o.e[a].c.x = 0.f;
+}
+__device__ __forceinline__ void clear_y(tf::PairTerms<float2> &o) {
+    o.phi.a.y = o.phi.b.y = o.phi.c.y = 0.f;
+#pragma unroll
+    for (int a = 0; a < 3; a++) o.e[a].a.y = o.e[a].b.y = o.e[a].c.y = 0.f;
+}
+
+// the sums of positions over 2^k and charges over 2^eq, and the FP64 pairs
+__device__ __forceinline__ double4 result(const tf::Acc<float2> (&A)[4], const double (&slow)[4], int k, int eq) {
+    double v[4];
+#pragma unroll
+    for (int c = 0; c < 4; c++)
+        v[c] = scalbn(((double)A[c].a.x + (double)A[c].a.y) +
+                          (((double)A[c].b.x + (double)A[c].b.y) + ((double)A[c].c.x + (double)A[c].c.y)),
+                      c ? eq - 2 * k : eq - k) +
+               slow[c];
+    return make_double4(v[0], v[1], v[2], v[3]);
+}
+
 // charges over 2^q_exponent in three floats, and the pair thresholds with the charges' own
 __global__ void __launch_bounds__(256)
 k_tf_charges(int64_t n, const double *__restrict__ q, const int *__restrict__ emax, const float *__restrict__ thr0,
              float *__restrict__ tq, float *__restrict__ thr) {
     const int e = q_exponent(*emax);
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const double s = scalbn(q[i], -e), as = fabs(s);
-        const bool ok = as == 0.0 || (as >= 0x1p-60 && as <= 1.0);  // NaN and infinities: no
-        const float a = ok ? (float)s : 0.f;
-        const double r = ok ? s - (double)a : 0.0;
-        const float b = (float)r;
-        tq[i] = a;
-        tq[n + i] = b;
-        tq[2 * n + i] = (float)(r - (double)b);
-        thr[i] = ok ? thr0[i] : __int_as_float(0x7f800000);
+        float f[3];
+        thr[i] = charge_split(q[i], e, thr0[i], f);
+#pragma unroll
+        for (int c = 0; c < 3; c++) tq[c * n + i] = f[c];
     }
 }
 
@@ -212,16 +241,12 @@ k_p2p_tf(int B, int64_t n, const double *__restrict__ x, const double *__restric
                     if (bx) {
                         // a target meets itself once: nothing, unless its charge is not finite
                         if (L.active && (bs + j0 != slot || isinf(th.x))) pair_f64(x, y, z, q, slot, bs + j0, slow);
-                        o.phi.a.x = o.phi.b.x = o.phi.c.x = 0.f;
-#pragma unroll
-                        for (int a = 0; a < 3; a++) o.e[a].a.x = o.e[a].b.x = o.e[a].c.x = 0.f;
+                        clear_x(o);
                     }
                     if (by) {
                         if (L.active && j0 + 1 < ns && (bs + j0 + 1 != slot || isinf(th.y)))
                             pair_f64(x, y, z, q, slot, bs + j0 + 1, slow);
-                        o.phi.a.y = o.phi.b.y = o.phi.c.y = 0.f;
-#pragma unroll
-                        for (int a = 0; a < 3; a++) o.e[a].a.y = o.e[a].b.y = o.e[a].c.y = 0.f;
+                        clear_y(o);
                     }
                 }
                 A[0].put(o.phi);
@@ -232,15 +257,7 @@ k_p2p_tf(int B, int64_t n, const double *__restrict__ x, const double *__restric
     }
     int k;
     grid_exponent(lo, hi, k);
-    const int eq = q_exponent(*emax);
-    double v[4];
-#pragma unroll
-    for (int c = 0; c < 4; c++)
-        v[c] = scalbn(((double)A[c].a.x + (double)A[c].a.y) +
-                          (((double)A[c].b.x + (double)A[c].b.y) + ((double)A[c].c.x + (double)A[c].c.y)),
-                      c ? eq - 2 * k : eq - k) +
-               slow[c];
-    double4 r = make_double4(v[0], v[1], v[2], v[3]);
+    double4 r = result(A, slow, k, q_exponent(*emax));
     const bool owner = L.combine(r, red);
     if (owner && part >= 0) {  // one segment of a split leaf: its partial sums
         partial[part + i] = r;
@@ -251,6 +268,242 @@ k_p2p_tf(int B, int64_t n, const double *__restrict__ x, const double *__restric
             field[3 * o] = (OutT)(far_E[slot] + r.y);
             field[3 * o + 1] = (OutT)(far_E[n + slot] + r.z);
             field[3 * o + 2] = (OutT)(far_E[2 * n + slot] + r.w);
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
+// The exact sum at selected targets (fmm_direct) in the same arithmetic. The
+// sources are split once into records of two (kRec float4: parts a, b, c of x,
+// y, z, q, then the thresholds; every lane of a warp reads the same record), a
+// slab of them at a time; a block takes 128 targets against a segment of the
+// slab and adds its sums to the (segment, target) slot; a last pass adds the
+// segments. 500k points, 1000 targets (5e8 pairs): one block per target in FP64
+// arithmetic (square root, two divisions and Neumaier sums a pair) 58.6 ms,
+// this 5.48 (85% of the FP32 pipe's rate for ~377 operations a pair); 1 target:
+// 8.40 -> 0.36 ms, 2000 points and 1000 targets 0.38 -> 0.08.
+// ---------------------------------------------------------------------------
+constexpr int kRec = 7;
+constexpr int64_t kSlab = 1 << 20;  // sources split at a time (58 MB of records)
+
+// the grid of the points: centre, 2^-k, whether it holds (grid_exponent), and the charges' exponent
+struct Grid {
+    double c[3], inv;
+    int k, ok, eq;
+    // a point's parts and its threshold on r^2
+    __device__ __forceinline__ float split(double x, double y, double z, float (&f)[3][3]) const {
+        bool exact = true;
+        const bool fine = ok && isfinite(x) && isfinite(y) && isfinite(z);
+        const double v[3] = {x, y, z};
+#pragma unroll
+        for (int a = 0; a < 3; a++) {
+            f[a][0] = f[a][1] = f[a][2] = 0.f;
+            if (fine) exact &= grid_split(v[a], c[a], inv, f[a]);
+        }
+        return !fine ? __int_as_float(0x7f800000) : exact ? kThrExact : kThrRounded;
+    }
+};
+
+struct DirectBox {  // the finite coordinates' range (order-preserving keys) and the largest charge's exponent
+    unsigned long long lo[3], hi[3];
+    int emax;
+    unsigned blocks;  // blocks done
+    Grid grid;        // from the last one
+};
+
+__global__ void k_direct_box_init(DirectBox *b) {
+    const int a = threadIdx.x;
+    if (a < 3) b->lo[a] = ~0ull, b->hi[a] = 0ull;
+    if (a == 0) b->emax = 0, b->blocks = 0;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(256)
+k_direct_box(const T *__restrict__ pts, const T *__restrict__ q, int64_t n, DirectBox *b) {
+    unsigned long long lo[3], hi[3];
+    int em = 0;
+#pragma unroll
+    for (int a = 0; a < 3; a++) lo[a] = ~0ull, hi[a] = 0ull;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+#pragma unroll
+        for (int a = 0; a < 3; a++) {
+            const double v = (double)pts[3 * i + a];
+            if (!isfinite(v)) continue;
+            const unsigned long long k = dkey(v);
+            lo[a] = min(lo[a], k);
+            hi[a] = max(hi[a], k);
+        }
+        const int e = (int)((__double_as_longlong((double)q[i]) >> 52) & 0x7ff);
+        if (e < 0x7ff) em = max(em, e);
+    }
+    em = __reduce_max_sync(0xffffffffu, em);
+#pragma unroll
+    for (int a = 0; a < 3; a++)
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            lo[a] = min(lo[a], __shfl_xor_sync(0xffffffffu, lo[a], o));
+            hi[a] = max(hi[a], __shfl_xor_sync(0xffffffffu, hi[a], o));
+        }
+    if ((threadIdx.x & 31) == 0) {
+#pragma unroll
+        for (int a = 0; a < 3; a++) {
+            atomicMin(&b->lo[a], lo[a]);
+            atomicMax(&b->hi[a], hi[a]);
+        }
+        if (em > 0) atomicMax(&b->emax, em);
+        __threadfence();
+    }
+    __syncthreads();
+    if (threadIdx.x == 0 && atomicAdd(&b->blocks, 1u) == gridDim.x - 1) {  // every block's part is in
+        __threadfence();
+        double l[3], h[3];
+        Grid G;
+        for (int a = 0; a < 3; a++) {
+            const unsigned long long kl = __ldcg(&b->lo[a]), kh = __ldcg(&b->hi[a]);
+            l[a] = kh ? dkey_inv(kl) : 0.0;  // no finite coordinate: an empty range at 0
+            h[a] = kh ? dkey_inv(kh) : 0.0;
+            G.c[a] = 0.5 * l[a] + 0.5 * h[a];
+        }
+        G.ok = grid_exponent(l, h, G.k);
+        G.inv = scalbn(1.0, -G.k);
+        G.eq = q_exponent(__ldcg(&b->emax));
+        b->grid = G;
+    }
+}
+
+template <typename T>
+__global__ void __launch_bounds__(256)
+k_direct_split(const T *__restrict__ pts, const T *__restrict__ q, int64_t n, int64_t j0, int64_t j1,
+               const DirectBox *__restrict__ box, float4 *__restrict__ rec) {
+    const Grid G = box->grid;
+    const int64_t m = (j1 - j0 + 1) & ~(int64_t)1;  // the last record is padded
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
+        float f[3][3] = {{1.f, 0.f, 0.f}, {0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}}, qf[3] = {0.f, 0.f, 0.f}, th = 0.f;
+        const int64_t j = j0 + i;
+        if (j < j1) {
+            th = G.split((double)pts[3 * j], (double)pts[3 * j + 1], (double)pts[3 * j + 2], f);
+            th = charge_split((double)q[j], G.eq, th, qf);
+        }
+        float *r = (float *)(rec + (i >> 1) * kRec) + (i & 1);
+#pragma unroll
+        for (int c = 0; c < 3; c++) {
+#pragma unroll
+            for (int a = 0; a < 3; a++) r[2 * (4 * c + a)] = -f[a][c];
+            r[2 * (4 * c + 3)] = qf[c];
+        }
+        r[24] = th;
+        r[26] = 0.f;
+    }
+}
+
+// source j on target i in FP64, pairs at zero distance skipped
+template <typename T>
+__device__ __noinline__ void direct_f64(const T *__restrict__ pts, const T *__restrict__ q, int64_t i, int64_t j,
+                                        double (&s)[4]) {
+    const double dx = (double)pts[3 * i] - (double)pts[3 * j], dy = (double)pts[3 * i + 1] - (double)pts[3 * j + 1],
+                 dz = (double)pts[3 * i + 2] - (double)pts[3 * j + 2];
+    const double r2 = dx * dx + dy * dy + dz * dz;
+    if (r2 == 0.0) return;
+    const double r = sqrt(r2), qj = (double)q[j], qr3 = qj / (r2 * r);
+    s[0] += qj / r;
+    s[1] += qr3 * dx;
+    s[2] += qr3 * dy;
+    s[3] += qr3 * dz;
+}
+
+// block (x: targets 128 x .., y: records [y len, (y + 1) len) of the slab)
+template <typename T>
+__global__ void __launch_bounds__(kT, 4)
+k_direct_tf(const T *__restrict__ pts, const T *__restrict__ q, int64_t n, const int64_t *__restrict__ targets,
+            int64_t nt, int64_t j0, int64_t j1, const DirectBox *__restrict__ box, const float4 *__restrict__ rec,
+            int64_t len, bool first, double4 *__restrict__ partial) {
+    __shared__ double4 red[kT];
+    const int64_t t0 = (int64_t)blockIdx.x * kT;
+    const P2PLane L((int)min((int64_t)kT, nt - t0), kT, threadIdx.x);
+    const int64_t i = L.active ? targets[t0 + L.target] : -1;
+    const bool on = i >= 0 && i < n;  // an index out of range: no access (the last pass writes NaN)
+    const bool busy = __any_sync(0xffffffffu, on);
+    float f[3][3] = {}, thr_i = 0.f;
+    if (on) thr_i = box->grid.split((double)pts[3 * i], (double)pts[3 * i + 1], (double)pts[3 * i + 2], f);
+    tf::Tri<float2> X[3];
+#pragma unroll
+    for (int a = 0; a < 3; a++)
+        X[a] = {make_float2(f[a][0], f[a][0]), make_float2(f[a][1], f[a][1]), make_float2(f[a][2], f[a][2])};
+    const float2 zero = make_float2(0.f, 0.f);
+    tf::Acc<float2> A[4] = {{zero, zero, zero}, {zero, zero, zero}, {zero, zero, zero}, {zero, zero, zero}};
+    double slow[4] = {0.0, 0.0, 0.0, 0.0};
+    const int64_t np = (j1 - j0 + 1) >> 1, p1 = busy ? min(np, (blockIdx.y + 1) * len) : 0;
+#pragma unroll 1
+    for (int64_t pp = blockIdx.y * len + L.slice; pp < p1; pp += L.slices) {
+        const float4 *r = rec + pp * kRec;
+        const float4 a0 = __ldg(r), a1 = __ldg(r + 1), b0 = __ldg(r + 2), b1 = __ldg(r + 3), c0 = __ldg(r + 4),
+                     c1 = __ldg(r + 5), th = __ldg(r + 6);
+        const tf::Tri<float2> Y[3] = {{make_float2(a0.x, a0.y), make_float2(b0.x, b0.y), make_float2(c0.x, c0.y)},
+                                      {make_float2(a0.z, a0.w), make_float2(b0.z, b0.w), make_float2(c0.z, c0.w)},
+                                      {make_float2(a1.x, a1.y), make_float2(b1.x, b1.y), make_float2(c1.x, c1.y)}};
+        const tf::Tri<float2> Q = {make_float2(a1.z, a1.w), make_float2(b1.z, b1.w), make_float2(c1.z, c1.w)};
+        tf::PairTerms<float2> o = tf::pair_terms(X, Y, Q);
+        const bool bx = o.r2.x < fmaxf(th.x, thr_i), by = o.r2.y < fmaxf(th.y, thr_i);
+        if (bx || by) {
+            const int64_t j = j0 + 2 * pp;
+            if (bx) {
+                if (on && (j != i || isinf(th.x))) direct_f64(pts, q, i, j, slow);
+                clear_x(o);
+            }
+            if (by) {
+                if (on && j + 1 < j1 && (j + 1 != i || isinf(th.y))) direct_f64(pts, q, i, j + 1, slow);
+                clear_y(o);
+            }
+        }
+        A[0].put(o.phi);
+#pragma unroll
+        for (int a = 0; a < 3; a++) A[1 + a].put(o.e[a]);
+    }
+    double4 r = result(A, slow, box->grid.k, box->grid.eq);
+    if (L.combine(r, red)) {
+        double4 *slot = partial + blockIdx.y * nt + t0 + L.target;
+        if (!first) {
+            const double4 o = *slot;
+            r.x += o.x;
+            r.y += o.y;
+            r.z += o.z;
+            r.w += o.w;
+        }
+        *slot = r;
+    }
+}
+
+template <typename T>
+__global__ void __launch_bounds__(256)
+k_direct_finish(int64_t n, const int64_t *__restrict__ targets, int64_t nt, int64_t segs,
+                const double4 *__restrict__ partial, T *__restrict__ pot, T *__restrict__ field) {
+    // a warp per target, the lanes over the segments
+    const int lane = threadIdx.x & 31;
+    for (int64_t t = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; t < nt;
+         t += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+        double4 r = make_double4(0.0, 0.0, 0.0, 0.0);
+        for (int64_t s = lane; s < segs; s += 32) {
+            const double4 o = partial[s * nt + t];
+            r.x += o.x;
+            r.y += o.y;
+            r.z += o.z;
+            r.w += o.w;
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            r.x += __shfl_xor_sync(0xffffffffu, r.x, o);
+            r.y += __shfl_xor_sync(0xffffffffu, r.y, o);
+            r.z += __shfl_xor_sync(0xffffffffu, r.z, o);
+            r.w += __shfl_xor_sync(0xffffffffu, r.w, o);
+        }
+        if (lane) continue;
+        const int64_t i = targets[t];
+        if (i < 0 || i >= n) r.x = r.y = r.z = r.w = __longlong_as_double(0x7ff8000000000000ll);
+        pot[t] = (T)r.x;
+        if (field) {
+            field[3 * t] = (T)r.y;
+            field[3 * t + 1] = (T)r.z;
+            field[3 * t + 2] = (T)r.w;
         }
     }
 }
@@ -286,6 +539,42 @@ cudaError_t tf_p2p(Plan &P, void *pot, void *field, int dtype) {
                    P.p2p_upart, P.p2p_nunits_dev, P.perm, P.far_phi, P.far_E, P.p2p_partial, (float *)pot,
                    (float *)field);
     return cudaGetLastError();
+}
+
+template <typename T>
+static cudaError_t direct_tf_run(const T *pts, const T *q, int64_t n, const int64_t *targets, int64_t nt, T *pot,
+                                 T *field, cudaStream_t st) {
+    // segments: enough blocks for about four waves of four per SM, 64 records at least
+    const int64_t slab = std::min(n, kSlab), recs = (slab + 1) / 2, tiles = (nt + kT - 1) / kT;
+    const int64_t want = std::max<int64_t>(1, 16 * (int64_t)sm_count() / tiles);
+    const int64_t len = std::max<int64_t>(64, (recs + want - 1) / want);
+    const int64_t segs = std::min<int64_t>((recs + len - 1) / len, 65535), len1 = (recs + segs - 1) / segs;
+    const size_t b0 = 512, b1 = (size_t)recs * kRec * 16, b2 = (size_t)segs * nt * sizeof(double4);
+    char *w = (char *)pool_alloc(b0 + ((b1 + 255) & ~(size_t)255) + b2, st);
+    if (!w) return cudaErrorMemoryAllocation;
+    DirectBox *box = (DirectBox *)w;
+    float4 *rec = (float4 *)(w + b0);
+    double4 *partial = (double4 *)(w + b0 + ((b1 + 255) & ~(size_t)255));
+    FMM_LAUNCH(k_direct_box_init, 1, 32, 0, st, box);
+    FMM_LAUNCH(k_direct_box<T>, grid_for(n), 256, 0, st, pts, q, n, box);
+    for (int64_t j0 = 0; j0 < n; j0 += kSlab) {
+        const int64_t j1 = std::min(n, j0 + kSlab);
+        FMM_LAUNCH(k_direct_split<T>, grid_for(j1 - j0), 256, 0, st, pts, q, n, j0, j1, box, rec);
+        FMM_LAUNCH(k_direct_tf<T>, dim3((unsigned)tiles, (unsigned)segs), kT, 0, st, pts, q, n, targets, nt, j0, j1,
+                   box, rec, len1, j0 == 0, partial);
+    }
+    FMM_LAUNCH(k_direct_finish<T>, grid_for(nt * 32), 256, 0, st, n, targets, nt, segs, partial, pot, field);
+    const cudaError_t e = cudaGetLastError();
+    pool_free(w, st);
+    return e;
+}
+
+// the exact sum; cudaErrorMemoryAllocation if its workspace cannot be had (nothing was launched then)
+cudaError_t direct_tf(const void *pts, const void *q, int64_t n, int dtype, const int64_t *targets, int64_t nt,
+                      void *pot, void *field, cudaStream_t st) {
+    if (dtype == FMM_F64)
+        return direct_tf_run((const double *)pts, (const double *)q, n, targets, nt, (double *)pot, (double *)field, st);
+    return direct_tf_run((const float *)pts, (const float *)q, n, targets, nt, (float *)pot, (float *)field, st);
 }
 
 }  // namespace fmm

@@ -62,3 +62,42 @@ def test_non_finite_charge_reaches_every_target(gpu_lib):
         plan = fmm.fmm_plan(torch.from_numpy(x).cuda(), 2, 2, 0.0)
         pot = fmm.fmm_eval(plan, torch.from_numpy(q).cuda())[0].cpu().numpy()
         assert not np.isfinite(pot).any()
+
+
+@pytest.mark.parametrize("nt", [1, 33, 129, 333])
+@pytest.mark.parametrize("kind", ["uniform", "close", "centre", "offset", "huge", "tiny", "charges", "plane"])
+def test_direct_matches_extended_precision(gpu_lib, kind, nt):
+    fmm = gpu_lib
+    x, q = cloud(kind, 333, np.random.default_rng(23))
+    t = np.arange(nt)[::-1].copy()
+    pot, fld = (v.cpu().numpy() for v in fmm.fmm_direct(torch.from_numpy(x).cuda(), torch.from_numpy(q).cuda(),
+                                                        torch.from_numpy(t).cuda()))
+    X, Q = x.astype(np.longdouble), q.astype(np.longdouble)
+    d = X[t][:, None, :] - X[None, :, :]
+    r = np.sqrt((d * d).sum(-1))
+    w = np.divide(np.longdouble(1), r, out=np.zeros_like(r), where=r > 0)
+    phi, mag = (w * Q).sum(1), (w * abs(Q)).sum(1)
+    E, magE = ((w ** 3 * Q)[:, :, None] * d).sum(1), (w ** 2 * abs(Q)).sum(1)
+    assert np.all(abs(pot - phi) <= 2.0 ** -49 * mag)
+    assert np.all(abs(fld - E) <= 2.0 ** -48 * magE[:, None])
+
+
+def test_direct_slabs_and_bad_indices(gpu_lib):
+    """More sources than one slab of records (2^20), float32, targets out of range and next to the slab's end."""
+    fmm = gpu_lib
+    n = (1 << 20) + 1001
+    rng = np.random.default_rng(5)
+    x, q = rng.random((n, 3)).astype(np.float32), rng.uniform(-1, 1, n).astype(np.float32)
+    t = np.array([0, -1, (1 << 20) - 1, 1 << 20, n, n - 1])
+    pot, fld = (v.cpu().numpy() for v in fmm.fmm_direct(torch.from_numpy(x).cuda(), torch.from_numpy(q).cuda(),
+                                                        torch.from_numpy(t).cuda()))
+    assert np.isnan(pot[[1, 4]]).all() and np.isnan(fld[[1, 4]]).all()
+    X, Q = x.astype(np.float64), q.astype(np.float64)
+    for k in (0, 2, 3, 5):
+        d = X[t[k]] - X
+        r = np.sqrt((d * d).sum(1))
+        w = np.divide(1.0, r, out=np.zeros_like(r), where=r > 0)
+        # float32 results: one rounding (2^-24) beside the reference's own 1e-12
+        assert abs(pot[k] - (w * Q).sum()) <= 2.0 ** -23 * abs((w * Q).sum()) + 1e-12 * (w * abs(Q)).sum()
+        E = ((w ** 3 * Q)[:, None] * d).sum(0)
+        assert np.all(abs(fld[k] - E) <= 2.0 ** -23 * abs(E) + 1e-12 * (w ** 2 * abs(Q)).sum())
