@@ -166,6 +166,7 @@ cudaError_t batch_setup(const Plan *const *plans, int n, const void *const *char
         y.charges = charges[i];
         y.pot = pot[i];
         y.field = field ? field[i] : nullptr;
+        if (y.field) R.fields = true;
         y.partial = P.p2p_partial;
         y.units = P.p2p_units;
         y.upart = P.p2p_upart;
@@ -300,10 +301,11 @@ cudaError_t batch_enqueue(const BatchRun &R, cudaStream_t st) {
         e = batch_l2l_down(R.S, G.off[kGrpL2L], n, G.blocks[kGrpL2L], G.p, G.tab, G.tab_df, R.next + g, st);
     }
     if (e == cudaSuccess) e = batch_l2p(R.S, R.off[kOffLeaf], n, R.blocks[kOffLeaf], R.pmax, st);
-    if (e == cudaSuccess) e = batch_p2p(R.S, R.units, R.usys, R.upart, R.nunits[0], kP2PTileSmall, R.dtype, st);
+    if (e == cudaSuccess) e = batch_p2p(R.S, R.units, R.usys, R.upart, R.nunits[0], kP2PTileSmall, R.dtype, R.fields,
+                                          st);
     if (e == cudaSuccess)
         e = batch_p2p(R.S, R.units + R.nunits[0], R.usys + R.nunits[0], R.upart + R.nunits[0], R.nunits[1], kP2PTile,
-                      R.dtype, st);
+                      R.dtype, R.fields, st);
     if (e == cudaSuccess) e = batch_combine(R.S, R.off[kOffComb], n, R.blocks[kOffComb], R.dtype, st);
     return e;
 }

@@ -358,7 +358,7 @@ cudaError_t batch_l2l_down(const BatchSys *S, const int32_t *off, int nsys, int6
                            const double *tab, const float2 *tab_df, unsigned long long *next, cudaStream_t st);
 cudaError_t batch_l2p(const BatchSys *S, const int32_t *off, int nsys, int64_t blocks, int pmax, cudaStream_t st);
 cudaError_t batch_p2p(const BatchSys *S, const int4 *units, const int32_t *usys, const int32_t *upart, int64_t n,
-                      int tile, int dtype, cudaStream_t st);
+                      int tile, int dtype, bool fields, cudaStream_t st);
 cudaError_t batch_combine(const BatchSys *S, const int32_t *off, int nsys, int64_t blocks, int dtype,
                           cudaStream_t st);
 cudaError_t batch_smem_limits(int p);
@@ -378,6 +378,7 @@ struct BatchGroup {
 struct BatchRun {
     void *mem = nullptr;
     int nsys = 0, pmax = 0, dtype = 0, ngroups = 0;
+    bool fields = false;     // some system has a field array
     BatchSys *S = nullptr;
     int32_t *off[4] = {};    // prepare, leaves (P2M, L2P), combine, unit merge
     int64_t blocks[4] = {};

@@ -17,6 +17,7 @@
 // O(1) whatever the box size.
 
 #include <algorithm>
+#include <type_traits>
 
 #include "fmm_internal.cuh"
 
@@ -336,6 +337,7 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __
 // B = (-z0, -z1, q0, q1), offsets from the target leaf's centre; the sums run
 // separately over even and odd sources.
 // far (cells apart): single-float offsets
+template <bool F>  // F: with the field
 __device__ __forceinline__ void far_pair2(float2 X, float2 Y, float2 Z, const float4 A, const float4 B,
                                           float2 *a) {
     const float2 dx = add2(X, make_float2(A.x, A.y));
@@ -343,33 +345,41 @@ __device__ __forceinline__ void far_pair2(float2 X, float2 Y, float2 Z, const fl
     const float2 dz = add2(Z, make_float2(B.x, B.y));
     const float2 r2 = fma2(dx, dx, fma2(dy, dy, mul2(dz, dz)));
     const float2 rinv = make_float2(rsqrt_ftz(r2.x), rsqrt_ftz(r2.y));
-    const float2 rinv2 = mul2(rinv, rinv);  // one packed product: fewer issue slots than two XU reciprocals
     const float2 qr = mul2(make_float2(B.z, B.w), rinv);
-    const float2 qr3 = mul2(qr, rinv2);
     a[0] = add2(a[0], qr);
-    a[1] = fma2(qr3, dx, a[1]);
-    a[2] = fma2(qr3, dy, a[2]);
-    a[3] = fma2(qr3, dz, a[3]);
+    if constexpr (F) {
+        const float2 rinv2 = mul2(rinv, rinv);  // one packed product: fewer issue slots than two XU reciprocals
+        const float2 qr3 = mul2(qr, rinv2);
+        a[1] = fma2(qr3, dx, a[1]);
+        a[2] = fma2(qr3, dy, a[2]);
+        a[3] = fma2(qr3, dz, a[3]);
+    }
 }
 
 // near (touching cells): split hi/lo offsets (lo parts staged as
 // C = (-xl0, -xl1, -yl0, -yl1), D = (-zl0, -zl1, ., .)), coincident points
-// skipped
+// skipped (their r^2 = 0 becomes infinite: 1/r and 1/r^2 are then zero)
+template <bool F>
 __device__ __forceinline__ void near_pair2(float2 X, float2 Y, float2 Z, float2 XL, float2 YL, float2 ZL,
                                            const float4 A, const float4 B, const float4 C, const float4 D,
                                            float2 *a) {
     const float2 dx = add2(add2(X, make_float2(A.x, A.y)), add2(XL, make_float2(C.x, C.y)));
     const float2 dy = add2(add2(Y, make_float2(A.z, A.w)), add2(YL, make_float2(C.z, C.w)));
     const float2 dz = add2(add2(Z, make_float2(B.x, B.y)), add2(ZL, make_float2(D.x, D.y)));
-    const float2 r2 = fma2(dx, dx, fma2(dy, dy, mul2(dz, dz)));
-    const float2 rinv = make_float2(r2.x > 0.f ? rsqrtf(r2.x) : 0.f, r2.y > 0.f ? rsqrtf(r2.y) : 0.f);
-    const float2 rinv2 = make_float2(r2.x > 0.f ? rcp_approx(r2.x) : 0.f, r2.y > 0.f ? rcp_approx(r2.y) : 0.f);
+    float2 r2 = fma2(dx, dx, fma2(dy, dy, mul2(dz, dz)));
+    const float inf = __int_as_float(0x7f800000);
+    r2.x = r2.x > 0.f ? r2.x : inf;
+    r2.y = r2.y > 0.f ? r2.y : inf;
+    const float2 rinv = make_float2(rsqrtf(r2.x), rsqrtf(r2.y));
     const float2 qr = mul2(make_float2(B.z, B.w), rinv);
-    const float2 qr3 = mul2(qr, rinv2);
     a[0] = add2(a[0], qr);
-    a[1] = fma2(qr3, dx, a[1]);
-    a[2] = fma2(qr3, dy, a[2]);
-    a[3] = fma2(qr3, dz, a[3]);
+    if constexpr (F) {
+        const float2 rinv2 = make_float2(rcp_approx(r2.x), rcp_approx(r2.y));
+        const float2 qr3 = mul2(qr, rinv2);
+        a[1] = fma2(qr3, dx, a[1]);
+        a[2] = fma2(qr3, dy, a[2]);
+        a[3] = fma2(qr3, dz, a[3]);
+    }
 }
 
 // exclusive prefix of v[0..len) in place (len <= kLeafChunk), the total at
@@ -427,7 +437,7 @@ __device__ __forceinline__ void block_excl_scan(int *v, int len, int *wsum) {
 // stream, 2T per pass. Per target the sources are summed in plain float over
 // runs of 64 (full runs with a fixed trip count) and the runs compensated
 // (Kahan).
-template <typename OutT, int T>
+template <typename OutT, int T, bool F>
 __device__ __forceinline__ void p2p_f32_body(int B, int64_t n, const float *__restrict__ hl,
                                              const float *__restrict__ qf, const int32_t *__restrict__ begin,
                                              const int32_t *__restrict__ count, const float4 *__restrict__ geo,
@@ -435,6 +445,7 @@ __device__ __forceinline__ void p2p_f32_body(int B, int64_t n, const float *__re
                                              const int32_t *__restrict__ perm, const float *__restrict__ far_phi,
                                              const float *__restrict__ far_E, double4 *__restrict__ partial,
                                              OutT *__restrict__ pot, OutT *__restrict__ field) {
+    constexpr int NA = F ? 4 : 1;  // sums: the potential, the field's components
     constexpr int kP2PThreads = T, kFarCap = 4 * T, kNearCap = 2 * T;
     __shared__ float4 sA[kFarCap / 2], sB[kFarCap / 2];    // hi parts and charges, per source pair
     __shared__ float4 sC[kNearCap / 2], sD[kNearCap / 2];  // lo parts (near leaves)
@@ -481,11 +492,11 @@ __device__ __forceinline__ void p2p_f32_body(int B, int64_t n, const float *__re
                 const int end = min(np, j0 + S * (kRun / 2));
                 float2 a[4];
 #pragma unroll
-                for (int c = 0; c < 4; c++) a[c] = make_float2(0.f, 0.f);
+                for (int c = 0; c < NA; c++) a[c] = make_float2(0.f, 0.f);
 #pragma unroll 4
-                for (int pp = j0 + slice; pp < end; pp += S) far_pair2(X, Y, Z, sA[pp], sB[pp], a);
+                for (int pp = j0 + slice; pp < end; pp += S) far_pair2<F>(X, Y, Z, sA[pp], sB[pp], a);
 #pragma unroll
-                for (int c = 0; c < 4; c++) kahan(sum[c], comp[c], a[c].x + a[c].y);
+                for (int c = 0; c < NA; c++) kahan(sum[c], comp[c], a[c].x + a[c].y);
             }
             return;
         }
@@ -494,16 +505,16 @@ __device__ __forceinline__ void p2p_f32_body(int B, int64_t n, const float *__re
             const int p0 = j0 >> 1;
             float2 a[4];
 #pragma unroll
-            for (int c = 0; c < 4; c++) a[c] = make_float2(0.f, 0.f);
+            for (int c = 0; c < NA; c++) a[c] = make_float2(0.f, 0.f);
             if (npair == kRun / 2) {
 #pragma unroll 8
-                for (int pp = 0; pp < kRun / 2; pp++) far_pair2(X, Y, Z, sA[p0 + pp], sB[p0 + pp], a);
+                for (int pp = 0; pp < kRun / 2; pp++) far_pair2<F>(X, Y, Z, sA[p0 + pp], sB[p0 + pp], a);
             } else {
 #pragma unroll 4
-                for (int pp = 0; pp < npair; pp++) far_pair2(X, Y, Z, sA[p0 + pp], sB[p0 + pp], a);
+                for (int pp = 0; pp < npair; pp++) far_pair2<F>(X, Y, Z, sA[p0 + pp], sB[p0 + pp], a);
             }
 #pragma unroll
-            for (int c = 0; c < 4; c++) kahan(sum[c], comp[c], a[c].x + a[c].y);
+            for (int c = 0; c < NA; c++) kahan(sum[c], comp[c], a[c].x + a[c].y);
         }
     };
     for (int cb = e0; cb < e1; cb += kLeafChunk) {
@@ -599,12 +610,12 @@ __device__ __forceinline__ void p2p_f32_body(int B, int64_t n, const float *__re
                     const int end = min(np, j0 + S * (kRun / 2));
                     float2 a[4];
 #pragma unroll
-                    for (int c = 0; c < 4; c++) a[c] = make_float2(0.f, 0.f);
+                    for (int c = 0; c < NA; c++) a[c] = make_float2(0.f, 0.f);
 #pragma unroll 2
                     for (int pp = j0 + slice; pp < end; pp += S)
-                        near_pair2(X, Y, Z, XL, YL, ZL, sA[pp], sB[pp], sC[pp], sD[pp], a);
+                        near_pair2<F>(X, Y, Z, XL, YL, ZL, sA[pp], sB[pp], sC[pp], sD[pp], a);
 #pragma unroll
-                    for (int c = 0; c < 4; c++) kahan(sum[c], comp[c], a[c].x + a[c].y);
+                    for (int c = 0; c < NA; c++) kahan(sum[c], comp[c], a[c].x + a[c].y);
                 }
                 continue;
             }
@@ -613,18 +624,18 @@ __device__ __forceinline__ void p2p_f32_body(int B, int64_t n, const float *__re
                 const int p0 = j0 >> 1;
                 float2 a[4];
 #pragma unroll
-                for (int c = 0; c < 4; c++) a[c] = make_float2(0.f, 0.f);
+                for (int c = 0; c < NA; c++) a[c] = make_float2(0.f, 0.f);
                 if (npair == kRun / 2) {
 #pragma unroll 8
                     for (int pp = 0; pp < kRun / 2; pp++)
-                        near_pair2(X, Y, Z, XL, YL, ZL, sA[p0 + pp], sB[p0 + pp], sC[p0 + pp], sD[p0 + pp], a);
+                        near_pair2<F>(X, Y, Z, XL, YL, ZL, sA[p0 + pp], sB[p0 + pp], sC[p0 + pp], sD[p0 + pp], a);
                 } else {
 #pragma unroll 4
                     for (int pp = 0; pp < npair; pp++)
-                        near_pair2(X, Y, Z, XL, YL, ZL, sA[p0 + pp], sB[p0 + pp], sC[p0 + pp], sD[p0 + pp], a);
+                        near_pair2<F>(X, Y, Z, XL, YL, ZL, sA[p0 + pp], sB[p0 + pp], sC[p0 + pp], sD[p0 + pp], a);
                 }
 #pragma unroll
-                for (int c = 0; c < 4; c++) kahan(sum[c], comp[c], a[c].x + a[c].y);
+                for (int c = 0; c < NA; c++) kahan(sum[c], comp[c], a[c].x + a[c].y);
             }
         }
     }
@@ -640,7 +651,7 @@ __device__ __forceinline__ void p2p_f32_body(int B, int64_t n, const float *__re
         const int64_t a = bt + io;
         const int64_t o = perm[a];
         pot[o] = (OutT)((double)far_phi[a] + v.x);
-        if (field) {
+        if (F && field) {  // (a system of a batch may have none)
             field[3 * o] = (OutT)((double)far_E[a] + v.y);
             field[3 * o + 1] = (OutT)((double)far_E[n + a] + v.z);
             field[3 * o + 2] = (OutT)((double)far_E[2 * n + a] + v.w);
@@ -658,7 +669,7 @@ __device__ __forceinline__ void p2p_f32_body(int B, int64_t n, const float *__re
 template <int T>
 constexpr int p2p_min_blocks(bool batched) { return T == kP2PTile ? 8 : batched ? 12 : 0; }
 
-template <typename OutT, int T>
+template <typename OutT, int T, bool F>
 __global__ void __launch_bounds__(T, p2p_min_blocks<T>(false))
 k_p2p_f32(int B, int64_t n, const float *__restrict__ hl, const float *__restrict__ qf,
           const int32_t *__restrict__ begin, const int32_t *__restrict__ count,
@@ -668,18 +679,18 @@ k_p2p_f32(int B, int64_t n, const float *__restrict__ hl, const float *__restric
           const float *__restrict__ far_E, double4 *__restrict__ partial, OutT *__restrict__ pot,
           OutT *__restrict__ field) {
     if ((int)blockIdx.x >= *nunits) return;  // launched for an upper bound on the units
-    p2p_f32_body<OutT, T>(B, n, hl, qf, begin, count, geo, ssrc, units[blockIdx.x], upart[blockIdx.x], perm,
+    p2p_f32_body<OutT, T, F>(B, n, hl, qf, begin, count, geo, ssrc, units[blockIdx.x], upart[blockIdx.x], perm,
                           far_phi, far_E, partial, pot, field);
 }
 
 // batched: the work units of every system in one list, heaviest first, each
 // with its system
-template <typename OutT, int T>
+template <typename OutT, int T, bool F>
 __global__ void __launch_bounds__(T, p2p_min_blocks<T>(true))
 k_b_p2p_f32(const BatchSys *__restrict__ S, const int4 *__restrict__ units, const int32_t *__restrict__ usys,
             const int32_t *__restrict__ upart) {
     const BatchSys &y = S[usys[blockIdx.x]];
-    p2p_f32_body<OutT, T>(y.B, y.n, y.hl, y.qf, y.begin, y.count, y.lgeo, y.ssrc, units[blockIdx.x],
+    p2p_f32_body<OutT, T, F>(y.B, y.n, y.hl, y.qf, y.begin, y.count, y.lgeo, y.ssrc, units[blockIdx.x],
                           upart[blockIdx.x], y.perm, y.far_phi, y.far_E, y.partial, (OutT *)y.pot, (OutT *)y.field);
 }
 
@@ -720,23 +731,37 @@ cudaError_t mixed_l2p(Plan &P) {
     return cudaGetLastError();
 }
 
-template <int T>
-static void launch_p2p_f32(Plan &P, void *pot, void *field, int dtype) {
+// f(integral constants): output type's size, tile, with the field
+template <typename Fn>
+static void p2p_instance(int dtype, int tile, bool fields, Fn &&f) {
+    auto by_field = [&](auto out, auto t) {
+        if (fields)
+            f(out, t, std::true_type{});
+        else
+            f(out, t, std::false_type{});
+    };
+    auto by_tile = [&](auto out) {
+        if (tile == kP2PTileSmall)
+            by_field(out, std::integral_constant<int, kP2PTileSmall>{});
+        else
+            by_field(out, std::integral_constant<int, kP2PTile>{});
+    };
     if (dtype == FMM_F64)
-        FMM_LAUNCH((k_p2p_f32<double, T>), (unsigned)P.p2p_nunits, T, 0, P.stream, P.B, P.n, P.hl, P.qf, P.begin,
-                   P.count, P.lgeo, P.ssrc[P.B], P.p2p_units, P.p2p_upart, P.p2p_nunits_dev, P.perm, P.far_phi_f,
-                   P.far_E_f, P.p2p_partial, (double *)pot, (double *)field);
+        by_tile(double{});
     else
-        FMM_LAUNCH((k_p2p_f32<float, T>), (unsigned)P.p2p_nunits, T, 0, P.stream, P.B, P.n, P.hl, P.qf, P.begin,
-                   P.count, P.lgeo, P.ssrc[P.B], P.p2p_units, P.p2p_upart, P.p2p_nunits_dev, P.perm, P.far_phi_f,
-                   P.far_E_f, P.p2p_partial, (float *)pot, (float *)field);
+        by_tile(float{});
 }
 
+// Without a field array only the potential is summed: 7 FP32 operations a
+// pair instead of 13.
 cudaError_t mixed_p2p(Plan &P, void *pot, void *field, int dtype) {
-    if (P.p2p_tile == kP2PTileSmall)
-        launch_p2p_f32<kP2PTileSmall>(P, pot, field, dtype);
-    else
-        launch_p2p_f32<kP2PTile>(P, pot, field, dtype);
+    p2p_instance(dtype, P.p2p_tile, field != nullptr, [&](auto out, auto tile, auto fld) {
+        using Out = decltype(out);
+        constexpr int T = decltype(tile)::value;
+        FMM_LAUNCH((k_p2p_f32<Out, T, decltype(fld)::value>), (unsigned)P.p2p_nunits, T, 0, P.stream, P.B, P.n, P.hl,
+                   P.qf, P.begin, P.count, P.lgeo, P.ssrc[P.B], P.p2p_units, P.p2p_upart, P.p2p_nunits_dev, P.perm,
+                   P.far_phi_f, P.far_E_f, P.p2p_partial, (Out *)pot, (Out *)field);
+    });
     return p2p_combine(P, pot, field, dtype);
 }
 
@@ -755,19 +780,13 @@ cudaError_t batch_l2p(const BatchSys *S, const int32_t *off, int nsys, int64_t b
 }
 
 cudaError_t batch_p2p(const BatchSys *S, const int4 *units, const int32_t *usys, const int32_t *upart, int64_t n,
-                      int tile, int dtype, cudaStream_t st) {
+                      int tile, int dtype, bool fields, cudaStream_t st) {
     if (n == 0) return cudaGetLastError();
-    if (tile == kP2PTileSmall) {
-        if (dtype == FMM_F64)
-            FMM_LAUNCH((k_b_p2p_f32<double, kP2PTileSmall>), (unsigned)n, kP2PTileSmall, 0, st, S, units, usys, upart);
-        else
-            FMM_LAUNCH((k_b_p2p_f32<float, kP2PTileSmall>), (unsigned)n, kP2PTileSmall, 0, st, S, units, usys, upart);
-    } else {
-        if (dtype == FMM_F64)
-            FMM_LAUNCH((k_b_p2p_f32<double, kP2PTile>), (unsigned)n, kP2PTile, 0, st, S, units, usys, upart);
-        else
-            FMM_LAUNCH((k_b_p2p_f32<float, kP2PTile>), (unsigned)n, kP2PTile, 0, st, S, units, usys, upart);
-    }
+    p2p_instance(dtype, tile, fields, [&](auto out, auto t, auto fld) {
+        constexpr int T = decltype(t)::value;
+        FMM_LAUNCH((k_b_p2p_f32<decltype(out), T, decltype(fld)::value>), (unsigned)n, T, 0, st, S, units, usys,
+                   upart);
+    });
     return cudaGetLastError();
 }
 

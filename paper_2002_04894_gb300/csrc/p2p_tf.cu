@@ -20,6 +20,7 @@
 // the charge is not finite or below 2^-60 of the largest.
 
 #include <algorithm>
+#include <type_traits>
 
 #include "fmm_internal.cuh"
 #include "trifloat.cuh"
@@ -155,7 +156,7 @@ __device__ __noinline__ void pair_f64(const double *__restrict__ x, const double
     s[3] += qr3 * dz;
 }
 
-template <typename OutT>
+template <typename OutT, bool F>  // F: with the field
 __global__ void __launch_bounds__(kT, 4)
 k_p2p_tf(int B, int64_t n, const double *__restrict__ x, const double *__restrict__ y, const double *__restrict__ z,
          const double *__restrict__ q, const float *__restrict__ pos, const float *__restrict__ tq,
@@ -234,7 +235,7 @@ k_p2p_tf(int B, int64_t n, const double *__restrict__ x, const double *__restric
                     {make_float2(a0.z, a0.w), make_float2(b0.z, b0.w), make_float2(c0.z, c0.w)},
                     {make_float2(a1.x, a1.y), make_float2(b1.x, b1.y), make_float2(c1.x, c1.y)}};
                 const tf::Tri<float2> Q = {make_float2(a1.z, a1.w), make_float2(b1.z, b1.w), make_float2(c1.z, c1.w)};
-                tf::PairTerms<float2> o = tf::pair_terms(X, Y, Q);
+                tf::PairTerms<float2> o = tf::pair_terms<float2, F>(X, Y, Q);
                 const bool bx = o.r2.x < fmaxf(th.x, thr_i), by = o.r2.y < fmaxf(th.y, thr_i);
                 if (bx || by) {
                     const int j0 = sb + 2 * pp;  // the leaf's sources j0 and j0 + 1 (padding past its last one)
@@ -251,7 +252,7 @@ k_p2p_tf(int B, int64_t n, const double *__restrict__ x, const double *__restric
                 }
                 A[0].put(o.phi);
 #pragma unroll
-                for (int a = 0; a < 3; a++) A[1 + a].put(o.e[a]);
+                for (int a = 0; a < (F ? 3 : 0); a++) A[1 + a].put(o.e[a]);
             }
         }
     }
@@ -264,7 +265,7 @@ k_p2p_tf(int B, int64_t n, const double *__restrict__ x, const double *__restric
     } else if (owner) {
         const int64_t o = perm[slot];
         pot[o] = (OutT)(far_phi[slot] + r.x);
-        if (field) {
+        if constexpr (F) {
             field[3 * o] = (OutT)(far_E[slot] + r.y);
             field[3 * o + 1] = (OutT)(far_E[n + slot] + r.z);
             field[3 * o + 2] = (OutT)(far_E[2 * n + slot] + r.w);
@@ -528,16 +529,17 @@ cudaError_t tf_p2p(Plan &P, void *pot, void *field, int dtype) {
     cudaMemsetAsync(P.tf_emax, 0, 4, P.stream);
     FMM_LAUNCH(k_tf_qmax, grid_for(P.n), 256, 0, P.stream, P.n, P.q, P.tf_emax);
     FMM_LAUNCH(k_tf_charges, grid_for(P.n), 256, 0, P.stream, P.n, P.q, P.tf_emax, P.tf_thr0, P.tf_q, P.tf_thr);
+    auto go = [&](auto out, auto fld) {  // without a field array only the potential is summed
+        using Out = decltype(out);
+        FMM_LAUNCH((k_p2p_tf<Out, decltype(fld)::value>), (unsigned)P.p2p_nunits, kT, 0, P.stream, P.B, P.n, P.x, P.y,
+                   P.z, P.q, P.tf_pos, P.tf_q, P.tf_thr0, P.tf_thr, P.lo, P.hi, P.tf_emax, P.begin, P.count,
+                   P.ssrc[P.B], P.p2p_units, P.p2p_upart, P.p2p_nunits_dev, P.perm, P.far_phi, P.far_E,
+                   P.p2p_partial, (Out *)pot, (Out *)field);
+    };
     if (dtype == FMM_F64)
-        FMM_LAUNCH(k_p2p_tf<double>, (unsigned)P.p2p_nunits, kT, 0, P.stream, P.B, P.n, P.x, P.y, P.z, P.q, P.tf_pos,
-                   P.tf_q, P.tf_thr0, P.tf_thr, P.lo, P.hi, P.tf_emax, P.begin, P.count, P.ssrc[P.B], P.p2p_units,
-                   P.p2p_upart, P.p2p_nunits_dev, P.perm, P.far_phi, P.far_E, P.p2p_partial, (double *)pot,
-                   (double *)field);
+        field ? go(double{}, std::true_type{}) : go(double{}, std::false_type{});
     else
-        FMM_LAUNCH(k_p2p_tf<float>, (unsigned)P.p2p_nunits, kT, 0, P.stream, P.B, P.n, P.x, P.y, P.z, P.q, P.tf_pos,
-                   P.tf_q, P.tf_thr0, P.tf_thr, P.lo, P.hi, P.tf_emax, P.begin, P.count, P.ssrc[P.B], P.p2p_units,
-                   P.p2p_upart, P.p2p_nunits_dev, P.perm, P.far_phi, P.far_E, P.p2p_partial, (float *)pot,
-                   (float *)field);
+        field ? go(float{}, std::true_type{}) : go(float{}, std::false_type{});
     return cudaGetLastError();
 }
 

@@ -134,7 +134,7 @@ struct PairTerms {
     Tri<V> phi, e[3];
 };
 
-template <class V>
+template <class V, bool F = true>  // F: with the field
 TF_DEV PairTerms<V> pair_terms(const Tri<V> (&x)[3], const Tri<V> (&ny)[3], const Tri<V> &q) {
     PairTerms<V> o;
     const Tri<V> d[3] = {diff(x[0], ny[0]), diff(x[1], ny[1]), diff(x[2], ny[2])};
@@ -196,6 +196,7 @@ TF_DEV PairTerms<V> pair_terms(const Tri<V> (&x)[3], const Tri<V> (&ny)[3], cons
         const V p = mul(Y.a, q.a);
         o.phi = product(Y, n0, nf, q, p, mul(p, cst(p, 0x1p-18f)));
     }
+    if constexpr (!F) return o;
     // 1 / r^2 = Z
     Tri<V> Z;
     {
