@@ -12,12 +12,12 @@
 // memory took 12,300).
 //
 // What bounds it: instruction issue of two warps per scheduler (255
-// registers), 60% busy, with the straight-line code (120 KB at p = 12) read
-// through the instruction caches by all warps in step, and the 32-lane sums
-// into the targets. 1.62e7 pairs of 2M Plummer points, 14 levels, M2L stage
-// before and now: p = 12 10.74 -> 5.37 ms, p = 10 6.91 -> 3.52, p = 8 4.39 ->
-// 2.01, p = 4 1.64 -> 0.72; odd orders (formerly tensor-core products) p = 9
-// 81.5 -> 2.89.
+// registers), over 60% busy, with the straight-line code (120 KB at p = 12)
+// read through the instruction caches, and the 32-lane sums into the targets
+// (0.9 of 5.4 ms). 1.62e7 pairs of 2M Plummer points, 14 levels, M2L stage
+// before and now: p = 12 10.74 -> 5.05 ms, p = 10 6.91 -> 3.32, p = 8 4.39 ->
+// 1.72, p = 4 1.64 -> 0.52; odd orders (formerly tensor-core products) p = 9
+// 81.5 -> 2.65.
 #pragma once
 
 #include <algorithm>
@@ -227,11 +227,15 @@ __device__ __forceinline__ void read_deg(const char *row, float (&r)[N + 1], flo
     }
 }
 
-// A block-wide barrier at the start of each large degree or order keeps the
-// warps of the SM within a few hundred instructions of each other, so that
-// the straight-line code is fetched once per SM and pass, not once per warp
-// (p = 12: 15.4 ms without the barriers, 5.5 with them, on 1.65e7 pairs).
-constexpr int kSyncFrom = 4;
+// Block-wide barriers at the start of the largest degrees and orders keep the
+// warps of the SM together on the longest straight-line code, so that it is
+// fetched once per SM and pass, not once per warp. Measured on 1.62e7 pairs
+// with barriers from degree 4 on / P - 2 / P - 1 / none: p = 12 5.36 / 5.05 /
+// 5.13 / 5.36 ms, p = 10 3.52 / 3.43 / 3.32 / 3.38, p = 8 2.01 / 1.97 / 1.85 /
+// 1.72, p = 6 1.25 / 1.22 / 1.14 / 0.91: the code of the orders below 10 fits
+// the instruction cache and the barriers only cost.
+template <int P>
+constexpr int sync_from() { return P >= 12 ? P - 2 : P >= 10 ? P - 1 : P + 1; }
 
 // forward rotation of degree N, scaled by (r_s / rho)^N
 template <int P, int N>
@@ -239,7 +243,7 @@ __device__ __forceinline__ void fwd(const char *rowp, const float2 *za, const fl
     constexpr int c0 = N * (N + 1) / 2;
     float ur[N + 1], ui[N + 1], xr[N + 1], xi[N + 1];
     read_deg<N>(rowp, ur, ui);
-    if constexpr (N >= kSyncFrom) __syncthreads();
+    if constexpr (N >= sync_from<P>()) __syncthreads();
     phase<N>(ur, ui, za);
     fold<kFwd1, N>(ur, ui, xr, xi);
     phase<N>(xr, xi, zb);
@@ -287,9 +291,9 @@ __host__ __device__ constexpr int group_first(int n) {  // first degree of degre
 
 // Column sums of degrees G..N over each of the warp's runs of equal target
 // (the pair list is sorted by target; `ends`: the runs' last lanes), added to
-// the run's target's scaled local in double. wt: the run's lanes as weights 0
-// or 1 (one run: all ones, set by the caller), so that a warp with several
-// targets costs a pass per run and not a loop over its lanes.
+// the run's target's scaled local in double. wt: of several runs, the lanes
+// of the present one as weights 0 or 1, so that a warp with several targets
+// costs a pass per run and not a loop over its lanes.
 template <int P, int G, int N>
 __device__ __forceinline__ void sum_group(const float *red, float *wt, int t32, unsigned ends,
                                           double2 *__restrict__ Lh) {
@@ -312,11 +316,20 @@ __device__ __forceinline__ void sum_group(const float *red, float *wt, int t32, 
             __syncwarp();
         }
         float2 a0 = make_float2(0.f, 0.f), a1 = make_float2(0.f, 0.f);
+        if (ends == 0x80000000u) {  // one target: no weights
 #pragma unroll
-        for (int i = 0; i < 8; i++) {
-            const float4 v = c4[i], u = w4[i];
-            a0 = __ffma2_rn(make_float2(v.x, v.y), make_float2(u.x, u.y), a0);
-            a1 = __ffma2_rn(make_float2(v.z, v.w), make_float2(u.z, u.w), a1);
+            for (int i = 0; i < 8; i++) {
+                const float4 v = c4[i];
+                a0 = __fadd2_rn(a0, make_float2(v.x, v.y));
+                a1 = __fadd2_rn(a1, make_float2(v.z, v.w));
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < 8; i++) {
+                const float4 v = c4[i], u = w4[i];
+                a0 = __ffma2_rn(make_float2(v.x, v.y), make_float2(u.x, u.y), a0);
+                a1 = __ffma2_rn(make_float2(v.z, v.w), make_float2(u.z, u.w), a1);
+            }
         }
         const float s = (a0.x + a0.y) + (a1.x + a1.y);
         if (on) atomicAdd(dst + (int64_t)t * (2 * NC), (double)s);
@@ -329,7 +342,7 @@ template <int P, int N>
 __device__ __forceinline__ void inv(State<P> &S, const float2 *za, const float2 *zb, float tp, float *red, float *wt,
                                     int t32, unsigned ends, double2 *__restrict__ Lh) {
     constexpr int c0 = N * (N + 1) / 2, G = group_first(N);
-    if constexpr (N >= kSyncFrom) __syncthreads();
+    if constexpr (N >= sync_from<P>()) __syncthreads();
     float ur[N + 1], ui[N + 1], xr[N + 1], xi[N + 1];
 #pragma unroll
     for (int m = 0; m <= N; m++) ur[m] = S.r[c0 + m] * tp, ui[m] = m ? S.i[c0 + m] * tp : 0.f;
@@ -489,7 +502,7 @@ __device__ __forceinline__ void run(Src &src, char *slice) {
         if (more) nxt = src.at(w0 + stride + (threadIdx.x >> 5));
         static_for<P + 1>([&](auto l) {
             constexpr int L = decltype(l)::value;
-            if constexpr (P - L >= kSyncFrom) __syncthreads();
+            if constexpr (P - L >= sync_from<P>()) __syncthreads();
             axial<P, L>(S);
             if constexpr (L == P / 6) {
                 if (more && !__any_sync(0xffffffffu, lost)) copy_rows<P>(src.Mf(nxt), nxt.gs, rowp, bar);
@@ -502,7 +515,6 @@ __device__ __forceinline__ void run(Src &src, char *slice) {
             float tp = cur.valid ? rinv : 0.f;
             const int up = __shfl_down_sync(0xffffffffu, cur.gt, 1);
             const unsigned ends = __ballot_sync(0xffffffffu, (threadIdx.x & 31) == 31 || up != cur.gt);
-            if (ends == 0x80000000u) wt[threadIdx.x & 31] = 1.f;
             double2 *Lh = src.Lh(cur);
             static_for<P + 1>([&](auto n) {
                 constexpr int N = decltype(n)::value;
