@@ -249,7 +249,7 @@ cudaError_t eval_downward(Plan &P) {
     stage_mark(P, FMM_STAGE_L2L, 0);
     // L2L into a level whose parents hold nothing would only add zeros
     if (one_launch_passes(P)) {
-        l2l_down(P, lw);
+        if (lw <= P.B || P.ext_active) l2l_down(P, lw);
     } else {
         for (int l = sp; l <= P.B; l += sp)
             if (l - sp >= lw || P.ext_active) l2l_level(P, l);

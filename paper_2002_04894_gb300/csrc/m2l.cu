@@ -2094,20 +2094,24 @@ cudaError_t m2l_f32_setup(Plan &P) {
 // single-precision M2L over all levels; leaves the unscaled result in L
 cudaError_t m2l_f32_all(Plan &P) {
     const int64_t total = P.nbox * P.nc;
+    const int64_t tot = total_weak(P);
+    if (tot == 0) {  // no pair reads a scaled multipole or leaves a scaled local
+        cudaMemsetAsync(P.L, 0, (size_t)total * sizeof(double2), P.stream);
+        return cudaGetLastError();
+    }
     const unsigned grid = (unsigned)std::min<int64_t>((P.nbox + 7) / 8, (int64_t)sm_count() * 16);  // 8 boxes (warps) per block
     FMM_LAUNCH(k_scale_multipoles, grid, 256, 0, P.stream, P.nbox, P.p, P.radius, P.M, P.Mf);
     cudaMemsetAsync(P.Lh, 0, (size_t)total * sizeof(double2), P.stream);
-    const int64_t tot = total_weak(P);
     cudaError_t e = cudaSuccess;
-    if (tot > 0 && P.m2l_tc) {
+    if (P.m2l_tc) {
         e = m2l_tc_launch(P);
-    } else if (tot > 0 && m2l_in_registers(P.p)) {
+    } else if (m2l_in_registers(P.p)) {
         const PairTable PT = pair_table(P);
         e = with_reg_order(P.p, [&](auto o) {
             reg::reg_launch<decltype(o)::value>(PT, tot, P.box_cf, P.Mf, P.Lh, P.d_err, P.stream);
             return cudaGetLastError();
         });
-    } else if (tot > 0) {
+    } else {
         switch (P.p) {
             case 14: e = launch_f32<14>(P, tot); break;
             case 16: e = launch_f32<16>(P, tot); break;
