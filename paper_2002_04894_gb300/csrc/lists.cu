@@ -231,6 +231,119 @@ __global__ void k_scan_add(int32_t *out, int64_t n, const int32_t *tile_sums) {
     if (i < n) out[i] += tile_sums[i / kScanTile];
 }
 
+// ---- the first levels in one block
+// The levels of up to kHeadBoxes boxes hold at most kHeadCand candidate pairs
+// (every pair of boxes), too few to be worth a launch sequence and a read-back
+// of the sizes each: one block takes them one after the other, the strong
+// list in shared memory, and the host reads all their sizes at once. 20k points,
+// 8 levels: list build 0.39 ms with every level launched by itself.
+constexpr int kHeadLevels = 6, kHeadBoxes = 1 << kHeadLevels, kHeadCand = kHeadBoxes * kHeadBoxes;
+constexpr int kHeadThreads = 1024, kHeadPer = kHeadCand / kHeadThreads;
+
+struct HeadLists {  // per level its arrays (of kHeadCand entries at most); level 0 has no weak ones
+    int32_t *wptr[kHeadLevels + 1], *sptr[kHeadLevels + 1];
+    int32_t *wsrc[kHeadLevels + 1], *wrow[kHeadLevels + 1], *ssrc[kHeadLevels + 1];
+    int32_t *srow;   // targets of the last level's strong pairs
+    int32_t *sizes;  // weak and strong pairs of each level
+};
+
+__global__ void __launch_bounds__(kHeadThreads)
+k_lists_head(int last, int step, double theta, const double *__restrict__ centre, const double *__restrict__ radius,
+             const float4 *__restrict__ cf, HeadLists H) {
+    __shared__ uint16_t src[kHeadCand], cs[kHeadCand], ct[kHeadCand];  // strong sources; the candidates' boxes
+    __shared__ uint16_t wpos[kHeadCand + 1];                            // weak candidates before each
+    __shared__ uint16_t ptr[2][kHeadBoxes + 1];                         // strong rows, this level's and the parent's
+    __shared__ unsigned wsum[kHeadThreads / 32];
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, C = 1 << step;
+    if (tid == 0) {
+        src[0] = 0;
+        ptr[0][0] = 0;
+        ptr[0][1] = 1;
+        H.wptr[0][0] = H.wptr[0][1] = 0;
+        H.sptr[0][0] = 0;
+        H.sptr[0][1] = 1;
+        H.ssrc[0][0] = 0;
+        H.sizes[0] = 0;
+        H.sizes[1] = 1;
+        if (last == 0) H.srow[0] = 0;
+    }
+    __syncthreads();
+    int cur = 0;
+    for (int l = step; l <= last; l += step, cur ^= 1) {
+        const uint16_t *pp = ptr[cur];
+        const int nT = 1 << (l - step), ncand = C * C * pp[nT], off = (1 << l) - 1;
+        // candidates of consecutive places per thread, in the order of k_cand:
+        // by target C T + a, then by source
+        unsigned weak = 0;
+#pragma unroll
+        for (int j = 0; j < kHeadPer; j++) {
+            const int c = tid * kHeadPer + j;
+            if (c >= ncand) break;
+            int lo = 0, hi = nT;  // C^2 pp[lo] <= c < C^2 pp[hi]
+            while (hi - lo > 1) {
+                const int mid = (lo + hi) >> 1;
+                if (C * C * pp[mid] <= c)
+                    lo = mid;
+                else
+                    hi = mid;
+            }
+            const int b0 = pp[lo], row = C * (pp[lo + 1] - b0), r = c - C * C * b0;
+            const int a = r / row, r2 = r - a * row;
+            const int t = C * lo + a, s = C * src[b0 + r2 / C] + r2 % C;
+            const int gt = off + t, gs = off + s;
+            int wk = theta > 0.0 ? theta_pretest((float)theta, cf[2 * gt], cf[2 * gt + 1], cf[2 * gs], cf[2 * gs + 1])
+                                 : 0;
+            if (wk < 0) wk = theta_weak(theta, centre + 3 * gt, radius[gt], centre + 3 * gs, radius[gs]) ? 1 : 0;
+            weak |= (unsigned)wk << j;
+            cs[c] = (uint16_t)s;
+            ct[c] = (uint16_t)t;
+        }
+        // exclusive scan of the weak counts
+        unsigned inc = __popc(weak);
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned y = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += y;
+        }
+        if (lane == 31) wsum[w] = inc;
+        __syncthreads();  // also: the parent's sources are read
+        unsigned run = inc - __popc(weak);
+        for (int i = 0; i < w; i++) run += wsum[i];
+#pragma unroll
+        for (int j = 0; j < kHeadPer; j++) {
+            const int c = tid * kHeadPer + j;
+            if (c >= ncand) break;
+            wpos[c] = (uint16_t)run;
+            if ((weak >> j) & 1u) {
+                H.wsrc[l][run] = cs[c];
+                H.wrow[l][run] = ct[c];
+                run++;
+            } else {
+                const int sp = c - (int)run;
+                src[sp] = cs[c];
+                H.ssrc[l][sp] = cs[c];
+                if (l + step > last) H.srow[sp] = ct[c];
+            }
+            if (c == ncand - 1) wpos[ncand] = (uint16_t)run;
+        }
+        __syncthreads();
+        const int nt = 1 << l;
+        for (int t = tid; t <= nt; t += kHeadThreads) {
+            const int T = t >> step, a = t & (C - 1);
+            const int first = t == nt ? ncand : C * C * pp[T] + a * C * (pp[T + 1] - pp[T]);
+            const int x = wpos[first];
+            H.wptr[l][t] = x;
+            H.sptr[l][t] = first - x;
+            ptr[cur ^ 1][t] = (uint16_t)(first - x);
+        }
+        if (tid == 0) {
+            H.sizes[2 * l] = wpos[ncand];
+            H.sizes[2 * l + 1] = ncand - wpos[ncand];
+        }
+        __syncthreads();
+    }
+}
+
 // per target leaf the near source points (sum of n_s over its strong leaf
 // pairs), and in total the sum over strong leaf pairs (t, s) of n_t * n_s.
 // Per leaf: its sources over the strong list, its number of near-field work
@@ -485,26 +598,43 @@ cudaError_t lists_build(Plan &P) {
     P.box_cf = (float4 *)palloc(P, (size_t)P.nbox * 2 * sizeof(float4));
     if (!P.box_cf) return cudaErrorMemoryAllocation;
     box_centres_f(P);
-    // level 0: the root is strongly connected to itself
-    P.wptr[0] = (int32_t *)palloc(P, 8);
-    P.sptr[0] = (int32_t *)palloc(P, 8);
-    P.ssrc[0] = (int32_t *)palloc(P, 4);
-    P.wsrc[0] = nullptr;
-    P.wrow[0] = nullptr;
-    int32_t *srow_prev = (int32_t *)dalloc(P, 4);
-    if (!P.wptr[0] || !P.sptr[0] || !P.ssrc[0] || !srow_prev) return cudaErrorMemoryAllocation;
-    const int32_t w0[2] = {0, 0}, s0[2] = {0, 1}, zero = 0;
-    cudaMemcpyAsync(P.wptr[0], w0, 8, cudaMemcpyHostToDevice, st);
-    cudaMemcpyAsync(P.sptr[0], s0, 8, cudaMemcpyHostToDevice, st);
-    cudaMemcpyAsync(P.ssrc[0], &zero, 4, cudaMemcpyHostToDevice, st);
-    cudaMemcpyAsync(srow_prev, &zero, 4, cudaMemcpyHostToDevice, st);
-    P.nweak[0] = 0;
-    P.nstrong[0] = 1;
     int32_t totals[2] = {0, 0};  // level sizes, read back synchronously
     cudaError_t e = cudaSuccess;
     const int step = P.step, C = 1 << step;
+    // level 0 (the root is strongly connected to itself) and the levels of few boxes
+    const int head = std::min(P.B, kHeadLevels) / step * step;
+    HeadLists H{};
+    H.srow = (int32_t *)dalloc(P, ((size_t)1 << (2 * head)) * 4);
+    H.sizes = (int32_t *)dalloc(P, 2 * (kHeadLevels + 1) * 4);
+    if (!H.srow || !H.sizes) return cudaErrorMemoryAllocation;
+    for (int l = 0; l <= head; l += step) {
+        const size_t nt = (size_t)1 << l, cap = nt * nt * 4;
+        P.wptr[l] = H.wptr[l] = (int32_t *)palloc(P, (nt + 1) * 4);
+        P.sptr[l] = H.sptr[l] = (int32_t *)palloc(P, (nt + 1) * 4);
+        P.ssrc[l] = H.ssrc[l] = (int32_t *)palloc(P, cap);
+        if (!P.wptr[l] || !P.sptr[l] || !P.ssrc[l]) return cudaErrorMemoryAllocation;
+        if (l == 0) continue;
+        P.wsrc[l] = H.wsrc[l] = (int32_t *)palloc(P, cap);
+        P.wrow[l] = H.wrow[l] = (int32_t *)palloc(P, cap);
+        if (!P.wsrc[l] || !P.wrow[l]) return cudaErrorMemoryAllocation;
+    }
+    FMM_LAUNCH(k_lists_head, 1, kHeadThreads, 0, st, head, step, P.theta, P.centre, P.radius, P.box_cf, H);
+    int32_t sizes[2 * (kHeadLevels + 1)] = {};
+    cudaMemcpyAsync(sizes, H.sizes, sizeof(sizes), cudaMemcpyDeviceToHost, st);
+    e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return e;
+    for (int l = 0; l <= head; l += step) {
+        if (l > 0 && (int64_t)C * C * P.nstrong[l - step] > g_list_capacity.load(std::memory_order_relaxed)) {
+            P.capacity_exceeded = true;
+            return cudaSuccess;
+        }
+        P.nweak[l] = sizes[2 * l];
+        P.nstrong[l] = sizes[2 * l + 1];
+    }
+    int32_t *srow_prev = H.srow;
     for (int l = 1; l <= P.B; l++) {
         const int64_t nt = (int64_t)1 << l;
+        if (l <= head && l % step == 0) continue;
         if (l % step) {
             // a bisection level inside a level of 2^step children: no pairs
             P.wptr[l] = (int32_t *)palloc(P, (nt + 1) * 4);
