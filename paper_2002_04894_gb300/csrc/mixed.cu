@@ -674,11 +674,12 @@ __device__ __forceinline__ void p2p_f32_body(int B, int64_t n, const float *__re
 // batched kernel holds the system's pointers in registers; at 64 registers for
 // 128-target tiles (8 blocks) and 80 for 64-target tiles (12 blocks) the
 // 512-system batch ran in 319.0 ms, against 324.8 ms at 80 registers for both
-// (328 ms at 72). The single-plan kernel takes 8 blocks for 128-target tiles
+// (328 ms at 72); since the tiles' last targets share threads, 9 blocks (56
+// registers): 48 systems 18.25 -> 17.93 ms (10 blocks 18.21). The single-plan kernel takes 8 blocks for 128-target tiles
 // (16.4 ms on 2M points; 16.9 with 7) and is left unconstrained for 64-target
 // tiles (61.2 ms on 8M points at 96 registers; 61.7 with 14 blocks).
 template <int T>
-constexpr int p2p_min_blocks(bool batched) { return T == kP2PTile ? 8 : batched ? 12 : 0; }
+constexpr int p2p_min_blocks(bool batched) { return T == kP2PTile ? (batched ? 9 : 8) : batched ? 12 : 0; }
 
 template <typename OutT, int T, bool F>
 __global__ void __launch_bounds__(T, p2p_min_blocks<T>(false))
