@@ -290,17 +290,6 @@ int fmm_plan(const void *points, int64_t n, int dtype, const fmm_opts *opts,
                      (size_t)P.nleaf * 2048 + (1 << 20);
     P.scratch.hint = (size_t)n * 40 + (size_t)P.nbox * 64 + (1 << 20);
 
-    // box point ranges depend on n and the level only
-    std::vector<int32_t> hb(P.nbox), hc(P.nbox);
-    hb[0] = 0;
-    hc[0] = (int32_t)n;
-    for (int64_t g = 0; g < P.nbox - P.nleaf; g++) {
-        const int32_t k = hc[g] / 2;
-        hb[2 * g + 1] = hb[g];
-        hc[2 * g + 1] = k;
-        hb[2 * g + 2] = hb[g] + k;
-        hc[2 * g + 2] = hc[g] - k;
-    }
     const size_t nb = (size_t)P.nbox;
     P.x = (double *)fmm::palloc(P, n * 8);
     P.y = (double *)fmm::palloc(P, n * 8);
@@ -322,8 +311,7 @@ int fmm_plan(const void *points, int64_t n, int dtype, const fmm_opts *opts,
         for (int s = 0; s < FMM_NSTAGES; s++)
             for (int k = 0; k < 2; k++)
                 if (cudaEventCreate(&P.ev[s][k]) != cudaSuccess) return fail(cuda_status(cudaGetLastError()));
-    cudaMemcpyAsync(P.begin, hb.data(), nb * 4, cudaMemcpyHostToDevice, P.stream);
-    cudaMemcpyAsync(P.count, hc.data(), nb * 4, cudaMemcpyHostToDevice, P.stream);
+    fmm::box_ranges(P);
     cudaMemsetAsync(P.plane, 0, nb * 8, P.stream);
     cudaMemsetAsync(P.d_err, 0, 16, P.stream);
 

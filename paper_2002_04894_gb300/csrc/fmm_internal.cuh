@@ -332,6 +332,8 @@ __device__ __forceinline__ double2 coef_at(const double2 *C, int n, int m) {
 // Host-side launchers (each in its own translation unit)
 // ---------------------------------------------------------------------------
 cudaError_t tree_build(Plan &P, const void *points_dev, int dtype);
+// every box's begin and count for median splits (they depend on n and the level only)
+void box_ranges(Plan &P);
 cudaError_t tight_geometry(Plan &P);
 cudaError_t lists_build(Plan &P);
 cudaError_t direct_run(const void *points, const void *charges, int64_t n, int dtype,

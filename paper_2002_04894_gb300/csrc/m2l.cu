@@ -29,6 +29,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstring>
 #include <atomic>
 #include <mutex>
 #include <vector>
@@ -1090,50 +1091,52 @@ cudaError_t allow_max_smem(const void *func, size_t need) {
     return cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize, room);
 }
 
-// the tables of order p, computed once per process (long double sums of
-// factorials: about a million operations at p = 12)
+// The tables of order p, computed once per process (long double sums of
+// factorials: about a million operations at p = 12), as doubles and then as
+// (hi, lo) float pairs for the double-float translations: one upload a plan.
 const std::vector<double> &m2l_tables_cached(int p) {
     static std::mutex mu;
     static std::vector<double> cache[FMM_MAX_P + 1];
     static bool ready[FMM_MAX_P + 1] = {};
     std::lock_guard<std::mutex> lock(mu);
     if (!ready[p]) {
-        cache[p] = m2l_tables(p);
+        const std::vector<double> t = m2l_tables(p);
+        std::vector<double> both(t);
+        for (double v : t) {
+            const float f[2] = {(float)v, (float)(v - (double)(float)v)};
+            double d;
+            std::memcpy(&d, f, 8);
+            both.push_back(d);
+        }
+        cache[p] = std::move(both);
         ready[p] = true;
     }
     return cache[p];
 }
 
 cudaError_t m2l_setup(Plan &P) {
-    const std::vector<double> &t = m2l_tables_cached(P.p);
-    P.m2l_ntab = (int)t.size();
-    P.m2l_tab = (double *)palloc(P, t.size() * 8);
+    const std::vector<double> &both = m2l_tables_cached(P.p);
+    const size_t nt = both.size() / 2, up = P.prec == FMM_PREC_MIXED ? 2 * nt : nt;
+    P.m2l_ntab = (int)nt;
+    P.m2l_tab = (double *)palloc(P, up * 8);
     P.m2m_arrive = (unsigned *)palloc(P, (size_t)P.nbox * 4);
     P.l2l_done = (int *)palloc(P, (size_t)P.nbox * 4);
     P.l2l_next = (unsigned long long *)palloc(P, 8);
     if (!P.m2l_tab || !P.m2m_arrive || !P.l2l_done || !P.l2l_next) return cudaErrorMemoryAllocation;
-    cudaError_t e = cudaMemcpyAsync(P.m2l_tab, t.data(), t.size() * 8, cudaMemcpyHostToDevice, P.stream);
-    if (e != cudaSuccess) return e;
     // stream-ordered copy from pageable memory completes before return
+    cudaError_t e = cudaMemcpyAsync(P.m2l_tab, both.data(), up * 8, cudaMemcpyHostToDevice, P.stream);
+    if (e != cudaSuccess) return e;
     if (P.prec == FMM_PREC_MIXED) {
-        // double-float translations: the tables as (hi, lo) float pairs, and
-        // the geometry of every box's translation to / from its parent
-        std::vector<float2> tdf(t.size());
-        for (size_t i = 0; i < t.size(); i++) {
-            const float h = (float)t[i];
-            tdf[i] = make_float2(h, (float)(t[i] - (double)h));
-        }
-        P.m2l_tab_df = (float2 *)palloc(P, tdf.size() * sizeof(float2));
+        // the pairs, and the geometry of every box's translation to / from its parent
+        P.m2l_tab_df = (float2 *)(P.m2l_tab + nt);
         P.box_geo = palloc(P, (size_t)P.nbox * sizeof(BoxGeo));
-        if (!P.m2l_tab_df || !P.box_geo) return cudaErrorMemoryAllocation;
-        e = cudaMemcpyAsync(P.m2l_tab_df, tdf.data(), tdf.size() * sizeof(float2), cudaMemcpyHostToDevice, P.stream);
-        if (e != cudaSuccess) return e;
+        if (!P.box_geo) return cudaErrorMemoryAllocation;
         FMM_LAUNCH(k_box_geo, (unsigned)std::min<int64_t>((P.nbox + 255) / 256, (int64_t)sm_count() * 8), 256, 0,
                    P.stream, P.nbox, P.step, P.centre, P.radius, (BoxGeo *)P.box_geo);
     }
     const int nc = P.nc;
     int threads = 64;
-    auto smem = [&](int T) { return (size_t)T * (nc + 2 * (P.p + 1)) * 16 + t.size() * 8; };
+    auto smem = [&](int T) { return (size_t)T * (nc + 2 * (P.p + 1)) * 16 + nt * 8; };
     if (smem(threads) > 220 * 1024) threads = 32;
     P.m2l_threads = threads;
     P.m2l_smem = smem(threads);

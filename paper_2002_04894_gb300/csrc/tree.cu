@@ -864,9 +864,37 @@ __global__ void k_children_eta(int level, int32_t *begin, int32_t *count, const 
 
 }  // namespace
 
+namespace {
+
+// box j of level l: the halvings of n that the bits of j select, high bit first
+__global__ void k_box_ranges(int64_t nbox, int32_t n, int32_t *__restrict__ begin, int32_t *__restrict__ count) {
+    for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < nbox; g += (int64_t)gridDim.x * blockDim.x) {
+        const unsigned long long h = (unsigned long long)(g + 1);  // a 1 bit, then the path from the root
+        int32_t b = 0, c = n;
+        for (int s = 62 - __clzll((long long)h); s >= 0; s--) {
+            const int32_t k = c / 2;
+            if ((h >> s) & 1ull)
+                b += k, c -= k;
+            else
+                c = k;
+        }
+        begin[g] = b;
+        count[g] = c;
+    }
+}
+
+}  // namespace
+
+// On the device: the host's loop over the boxes and the upload of its arrays
+// took longer than the small levels of the tree.
+void box_ranges(Plan &P) {
+    FMM_LAUNCH(k_box_ranges, (unsigned)std::min<int64_t>((P.nbox + 255) / 256, (int64_t)sm_count() * 8), 256, 0,
+               P.stream, P.nbox, (int32_t)P.n, P.begin, P.count);
+}
+
 // Builds the tree: points (device, n x 3, dtype) -> leaf-order SoA positions,
-// permutation, and all box cells/geometry. Box begin/count are host-computed
-// (they depend on n and the level only) and already on the device.
+// permutation, and all box cells/geometry. Box begin/count (box_ranges) are
+// already there.
 cudaError_t tree_build(Plan &P, const void *pts, int dtype) {
     const int64_t n = P.n;
     cudaStream_t st = P.stream;
@@ -888,8 +916,8 @@ cudaError_t tree_build(Plan &P, const void *pts, int dtype) {
         return cudaErrorMemoryAllocation;
     cudaMemsetAsync(arrived, 0, (size_t)maxseg * 4, st);
 
-    unsigned long long init[6] = {~0ull, ~0ull, ~0ull, 0ull, 0ull, 0ull};
-    cudaMemcpyAsync(bbox, init, sizeof(init), cudaMemcpyHostToDevice, st);
+    cudaMemsetAsync(bbox, 0xff, 24, st);  // minima
+    cudaMemsetAsync(bbox + 3, 0, 24, st);
     const int pgrid = (int)std::min<int64_t>((n + kThreads - 1) / kThreads, (int64_t)sm_count() * 8);
     if (dtype == FMM_F64)
         FMM_LAUNCH(k_prepare<double>, pgrid, kThreads, 0, st, (const double *)pts, n, P.x, P.y, P.z,
