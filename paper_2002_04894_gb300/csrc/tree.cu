@@ -1056,11 +1056,15 @@ cudaError_t tree_build(Plan &P, const void *pts, int dtype) {
             cudaMemsetAsync(dmax, 0, 4, st);
             FMM_LAUNCH(k_children_eta, sg, 128, 0, st, l, P.begin, P.count, ksplit, splane, P.lo, P.hi,
                                                             P.centre, P.radius, P.axis, P.plane, dmax);
-            int hmax = 0;
-            cudaMemcpyAsync(&hmax, dmax, 4, cudaMemcpyDeviceToHost, st);
-            const cudaError_t es = cudaStreamSynchronize(st);
-            if (es != cudaSuccess) return es;
-            maxn = hmax;
+            // the next level's regime goes by its largest box; below the small
+            // regime's limit it stays there, whatever the sizes
+            if (maxn > kSmallCap) {
+                int hmax = 0;
+                cudaMemcpyAsync(&hmax, dmax, 4, cudaMemcpyDeviceToHost, st);
+                const cudaError_t es = cudaStreamSynchronize(st);
+                if (es != cudaSuccess) return es;
+                maxn = hmax;
+            }
         }
         std::swap(xa, xb);
         std::swap(ya, yb);
