@@ -21,7 +21,7 @@ constexpr int kP2PTileSmall = 64;
 // strong list holds more is cut into segments, each its own unit
 constexpr int kP2PSegSources = 1 << 16;
 // few leaves: units per SM to cut their lists for, and the shortest segment
-constexpr int kP2PUnitsPerSM = 10, kP2PSegMin = 256;
+constexpr int kP2PUnitsPerSM = 10, kP2PSegMin = 128;
 
 // ---------------------------------------------------------------------------
 // Plan: everything lives in device memory owned by the plan.
