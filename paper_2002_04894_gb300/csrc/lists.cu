@@ -189,6 +189,7 @@ __device__ int32_t block_exclusive(int32_t v, int32_t *total) {
 
 __global__ void __launch_bounds__(kScanThreads)
 k_scan_tiles(const int32_t *in, int32_t *out, int64_t n, int32_t *tile_sums) {
+    // tile_sums[tile] = its sum (one tile: the total, at out[n])
     __shared__ int32_t tot;
     const int64_t base = blockIdx.x * (int64_t)kScanTile + threadIdx.x * kScanItems;
     int32_t v[kScanItems], s = 0;
@@ -204,26 +205,6 @@ k_scan_tiles(const int32_t *in, int32_t *out, int64_t n, int32_t *tile_sums) {
         run += v[j];
     }
     if (threadIdx.x == 0) tile_sums[blockIdx.x] = tot;
-}
-
-__global__ void __launch_bounds__(kScanThreads)
-k_scan_sums(int32_t *tile_sums, int64_t ntiles, int32_t *total_out) {
-    // single block; ntiles <= kScanTile
-    __shared__ int32_t tot;
-    const int64_t base = threadIdx.x * (int64_t)kScanItems;
-    int32_t v[kScanItems], s = 0;
-#pragma unroll
-    for (int j = 0; j < kScanItems; j++) {
-        v[j] = base + j < ntiles ? tile_sums[base + j] : 0;
-        s += v[j];
-    }
-    int32_t run = block_exclusive(s, &tot);
-#pragma unroll
-    for (int j = 0; j < kScanItems; j++) {
-        if (base + j < ntiles) tile_sums[base + j] = run;
-        run += v[j];
-    }
-    if (threadIdx.x == 0) *total_out = tot;
 }
 
 __global__ void k_scan_add(int32_t *out, int64_t n, const int32_t *tile_sums) {
@@ -553,10 +534,7 @@ cudaError_t scan_exclusive(Plan &P, const int32_t *in, int32_t *out, int64_t n) 
     }
     const int64_t ntiles = (n + kScanTile - 1) / kScanTile;
     if (ntiles == 1) {
-        int32_t *sums = (int32_t *)dalloc(P, 4);
-        if (!sums) return cudaErrorMemoryAllocation;
-        FMM_LAUNCH(k_scan_tiles, 1, kScanThreads, 0, P.stream, in, out, n, sums);
-        FMM_LAUNCH(k_scan_sums, 1, kScanThreads, 0, P.stream, sums, 1, out + n);
+        FMM_LAUNCH(k_scan_tiles, 1, kScanThreads, 0, P.stream, in, out, n, out + n);
         return cudaGetLastError();
     }
     // tile sums -> their exclusive scan (recursively) -> add back

@@ -74,6 +74,31 @@ __device__ void box_geometry(double *lo, double *hi, double *centre, double *rad
     axis[g] = ax;
 }
 
+// The cells' arrays, for the kernels that write a split box's children.
+struct Cells {
+    double *lo = nullptr, *hi = nullptr, *centre = nullptr, *radius = nullptr, *plane = nullptr;
+    int32_t *axis = nullptr;
+};
+
+// The plane of box g's median split: halfway between the largest left and the
+// smallest right coordinate (v, minr: their keys); of one point its
+// coordinate (v), of none the cell's midpoint.
+__device__ __forceinline__ double median_plane(int n, uint64_t v, uint64_t minr, double lo, double hi) {
+    if (n >= 2) return __dmul_rn(0.5, __dadd_rn(dkey_inv(v), dkey_inv(minr)));
+    return n == 1 ? dkey_inv(v) : __dmul_rn(0.5, __dadd_rn(lo, hi));
+}
+
+// Child `side` (0 left, 1 right) of box g cut at sp along axis ax; the left one's caller also stores the plane.
+__device__ __forceinline__ void make_child(const Cells &c, int64_t g, int ax, double sp, int side) {
+    const int64_t ch = 2 * g + 1 + side;
+    if (side == 0) c.plane[g] = sp;
+    for (int d = 0; d < 3; d++) {
+        c.lo[3 * ch + d] = side == 1 && d == ax ? sp : c.lo[3 * g + d];
+        c.hi[3 * ch + d] = side == 0 && d == ax ? sp : c.hi[3 * g + d];
+    }
+    box_geometry(c.lo, c.hi, c.centre, c.radius, c.axis, ch);
+}
+
 // --------------------------------------------------------------------------
 // Input: n x 3 row-major -> SoA doubles, -0.0 -> +0.0, finiteness, bounding box
 // --------------------------------------------------------------------------
@@ -184,6 +209,7 @@ __device__ __forceinline__ bool prefix_match(uint64_t key, uint64_t prefix, int 
 // --------------------------------------------------------------------------
 // Small regime: one CTA per box
 // --------------------------------------------------------------------------
+template <bool kKids>  // writes the children's cells
 __global__ void __launch_bounds__(kThreads)
 k_split_small(int level, const double *__restrict__ xin, const double *__restrict__ yin,
               const double *__restrict__ zin, const int32_t *__restrict__ iin,
@@ -191,7 +217,7 @@ k_split_small(int level, const double *__restrict__ xin, const double *__restric
               int32_t *__restrict__ iout, const int32_t *__restrict__ begin,
               const int32_t *__restrict__ count, const int32_t *__restrict__ axis,
               uint64_t *sel_v, unsigned long long *sel_minr, int *err,
-              const unsigned long long *__restrict__ thr, int32_t *__restrict__ ksplit) {
+              const unsigned long long *__restrict__ thr, int32_t *__restrict__ ksplit, Cells cells) {
     // thr == nullptr: median split (left = floor(n/2) smallest keys);
     // otherwise threshold split (left = keys below thr[s], count to ksplit[s])
     __shared__ uint64_t keys[kSmallCap];
@@ -224,6 +250,10 @@ k_split_small(int level, const double *__restrict__ xin, const double *__restric
             }
         }
         if (n == 0 && thr && tid == 0) ksplit[s] = 0;
+        if (kKids && lane == 0 && w < 2) {
+            const uint64_t v1 = n ? dkey(src[b]) : 0;
+            make_child(cells, g, ax, median_plane(n, v1, v1, cells.lo[3 * g + ax], cells.hi[3 * g + ax]), w);
+        }
         return;
     }
     for (int i = tid; i < n; i += kThreads) keys[i] = dkey(src[b + i]);
@@ -330,10 +360,12 @@ k_split_small(int level, const double *__restrict__ xin, const double *__restric
         }
         lrun += __popc(fm);
     }
+    const unsigned long long right = eqtot > need_eq ? (unsigned long long)v : s_minr;
     if (tid == 0 && !thr) {
         sel_v[s] = v;
-        sel_minr[s] = eqtot > need_eq ? (unsigned long long)v : s_minr;
+        sel_minr[s] = right;
     }
+    if (kKids && lane == 0 && w < 2) make_child(cells, g, ax, median_plane(n, v, right, 0.0, 0.0), w);
 }
 
 // --------------------------------------------------------------------------
@@ -352,14 +384,16 @@ constexpr int kClThreads = 1024, kClWarps = kClThreads / 32;
 constexpr int kClKeys = 16384;      // keys of a CTA at most (128 KB)
 constexpr int kClMax = 8;           // CTAs of a cluster (the portable limit)
 constexpr int kMidCap = kClKeys * kClMax;
+constexpr int kFewBoxes = 1024;
 
+template <bool kKids>
 __global__ void __launch_bounds__(kClThreads)
 k_split_cluster(int level, const double *__restrict__ xin, const double *__restrict__ yin,
                 const double *__restrict__ zin, const int32_t *__restrict__ iin, double *__restrict__ xout,
                 double *__restrict__ yout, double *__restrict__ zout, int32_t *__restrict__ iout,
                 const int32_t *__restrict__ begin, const int32_t *__restrict__ count,
                 const int32_t *__restrict__ axis, uint64_t *sel_v, unsigned long long *sel_minr, int *err,
-                const unsigned long long *__restrict__ thr, int32_t *__restrict__ ksplit) {
+                const unsigned long long *__restrict__ thr, int32_t *__restrict__ ksplit, Cells cells) {
     // thr as for k_split_small
     namespace cg = cooperative_groups;
     extern __shared__ uint64_t keys[];  // this CTA's, kClKeys
@@ -396,6 +430,10 @@ k_split_cluster(int level, const double *__restrict__ xin, const double *__restr
             } else if (thr) {
                 ksplit[s] = 0;
             }
+        }
+        if (kKids && r == 0 && lane == 0 && w < 2) {
+            const uint64_t v1 = n ? dkey(src[b]) : 0;
+            make_child(cells, g, ax, median_plane(n, v1, v1, cells.lo[3 * g + ax], cells.hi[3 * g + ax]), w);
         }
         return;
     }
@@ -533,10 +571,12 @@ k_split_cluster(int level, const double *__restrict__ xin, const double *__restr
         }
         lrun += __popc(fm);
     }
+    const unsigned long long right = eqtot > need_eq ? (unsigned long long)v : minr;
     if (r == 0 && tid == 0 && !thr) {
         sel_v[s] = v;
-        sel_minr[s] = eqtot > need_eq ? (unsigned long long)v : minr;
+        sel_minr[s] = right;
     }
+    if (kKids && r == 0 && lane == 0 && w < 2) make_child(cells, g, ax, median_plane(n, v, right, 0.0, 0.0), w);
 }
 
 // --------------------------------------------------------------------------
@@ -788,26 +828,11 @@ __global__ void k_children(int level, const int32_t *count, const uint64_t *sel_
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= (1 << level)) return;
     const int64_t g = ((int64_t)1 << level) - 1 + s;
-    const int n = count[g], ax = axis[g];
-    double sp;
-    if (n >= 2)
-        sp = __dmul_rn(0.5, __dadd_rn(dkey_inv(sel_v[s]), dkey_inv(sel_minr[s])));
-    else if (n == 1)
-        sp = dkey_inv(sel_minr[s]);
-    else
-        sp = __dmul_rn(0.5, __dadd_rn(lo[3 * g + ax], hi[3 * g + ax]));
-    plane[g] = sp;
-    const int64_t a = 2 * g + 1, c = 2 * g + 2;
-    for (int d = 0; d < 3; d++) {
-        lo[3 * a + d] = lo[3 * g + d];
-        hi[3 * a + d] = hi[3 * g + d];
-        lo[3 * c + d] = lo[3 * g + d];
-        hi[3 * c + d] = hi[3 * g + d];
-    }
-    hi[3 * a + ax] = sp;
-    lo[3 * c + ax] = sp;
-    box_geometry(lo, hi, centre, radius, axis, a);
-    box_geometry(lo, hi, centre, radius, axis, c);
+    const int ax = axis[g];
+    const double sp = median_plane(count[g], sel_v[s], sel_minr[s], lo[3 * g + ax], hi[3 * g + ax]);
+    const Cells c{lo, hi, centre, radius, plane, axis};
+    make_child(c, g, ax, sp, 0);
+    make_child(c, g, ax, sp, 1);
 }
 
 // eta in [0,1): the plane s = eta * median plane + (1 - eta) * cell midpoint
@@ -952,12 +977,20 @@ cudaError_t tree_build(Plan &P, const void *pts, int dtype) {
         const int S = 1 << l;
         const unsigned sg = (unsigned)((S + 127) / 128);
         if (!eta_mode) maxn = (n + S - 1) / S;
+        // A median split's own kernel writes the children's cells where the
+        // boxes are few: a launch less (20k points, 8 levels: tree 0.181 ->
+        // 0.144 ms). With many boxes the square roots at the end of every CTA
+        // cost more than a kernel for all of them (8M points: 5.35 against 4.98).
+        const bool with_children = !eta_mode && maxn <= kMidCap && S <= kFewBoxes;
         if (maxn <= kMidCap) {
             // one CTA or one cluster per box, by the largest box
+            const auto small = with_children ? k_split_small<true> : k_split_small<false>;
+            const auto cluster = with_children ? k_split_cluster<true> : k_split_cluster<false>;
+            const Cells cells = with_children ? Cells{P.lo, P.hi, P.centre, P.radius, P.plane, P.axis} : Cells{};
             auto split = [&](const unsigned long long *t, int32_t *ks) -> cudaError_t {
                 if (maxn <= kSmallCap) {
-                    FMM_LAUNCH(k_split_small, S, kThreads, 0, st, l, xa, ya, za, ia, xb, yb, zb, ib, P.begin, P.count,
-                               P.axis, sel_v, sel_minr, P.d_err, t, ks);
+                    FMM_LAUNCH(small, S, kThreads, 0, st, l, xa, ya, za, ia, xb, yb, zb, ib, P.begin, P.count, P.axis,
+                               sel_v, sel_minr, P.d_err, t, ks, cells);
                     return cudaGetLastError();
                 }
                 // as few CTAs as hold the largest box, more while SMs are left over
@@ -977,14 +1010,14 @@ cudaError_t tree_build(Plan &P, const void *pts, int dtype) {
                 cfg.attrs = at;
                 cfg.numAttrs = 1;
                 const cudaError_t e = cudaLaunchKernelEx(
-                    &cfg, k_split_cluster, l, (const double *)xa, (const double *)ya, (const double *)za,
+                    &cfg, cluster, l, (const double *)xa, (const double *)ya, (const double *)za,
                     (const int32_t *)ia, xb, yb, zb, ib, (const int32_t *)P.begin, (const int32_t *)P.count,
-                    (const int32_t *)P.axis, sel_v, sel_minr, P.d_err, t, ks);
+                    (const int32_t *)P.axis, sel_v, sel_minr, P.d_err, t, ks, cells);
                 g_launches.fetch_add(1, std::memory_order_relaxed);
                 return e;
             };
             cudaError_t es = cudaSuccess;
-            if (maxn > kSmallCap) es = allow_max_smem((const void *)k_split_cluster, kClKeys * sizeof(uint64_t));
+            if (maxn > kSmallCap) es = allow_max_smem((const void *)cluster, kClKeys * sizeof(uint64_t));
             if (es == cudaSuccess && need_median) es = split(nullptr, nullptr);
             if (es == cudaSuccess && eta_mode) {
                 FMM_LAUNCH(k_eta_plane, sg, 128, 0, st, l, P.eta, P.count, P.axis, P.lo, P.hi, sel_v,
@@ -1049,7 +1082,9 @@ cudaError_t tree_build(Plan &P, const void *pts, int dtype) {
                                                          (const int32_t *)ksplit);
             }
         }
-        if (!eta_mode) {
+        if (with_children) {
+            // written above
+        } else if (!eta_mode) {
             FMM_LAUNCH(k_children, sg, 128, 0, st, l, P.count, sel_v, sel_minr, P.lo, P.hi, P.centre,
                                                         P.radius, P.axis, P.plane);
         } else {
@@ -1351,10 +1386,9 @@ extern "C" int fmm_orb_order_noalloc(const void *points, int64_t n, int dtype, i
     FMM_LAUNCH(k_root, 1, 32, 0, st, bbox, RootCell{}, lo, hi, centre, radius, axis, err);
     for (int l = 0; l < levels; l++) {
         const int S = 1 << l;
-        FMM_LAUNCH(k_split_small, S, kThreads, 0, st, l, xa, ya, za, ia, xb, yb, zb, ib, begin, count,
-                   axis, sel_v, sel_minr, err, (const unsigned long long *)nullptr, (int32_t *)nullptr);
-        FMM_LAUNCH(k_children, (S + 127) / 128, 128, 0, st, l, count, sel_v, sel_minr, lo, hi, centre,
-                   radius, axis, plane);
+        FMM_LAUNCH(k_split_small<true>, S, kThreads, 0, st, l, xa, ya, za, ia, xb, yb, zb, ib, begin, count,
+                   axis, sel_v, sel_minr, err, (const unsigned long long *)nullptr, (int32_t *)nullptr,
+                   Cells{lo, hi, centre, radius, plane, axis});
         std::swap(xa, xb);
         std::swap(ya, yb);
         std::swap(za, zb);
