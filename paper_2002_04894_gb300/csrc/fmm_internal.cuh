@@ -219,8 +219,7 @@ struct Plan {
     unsigned *m2m_arrive = nullptr;         // one-launch upward pass: arrivals per parent
     int *l2l_done = nullptr;                // one-launch downward pass: box finished
     unsigned long long *l2l_next = nullptr; // one-launch downward pass: next box to take
-    int m2l_ntab = 0, m2l_threads = 0;
-    size_t m2l_smem = 0;
+    int m2l_ntab = 0, m2l_warps = 0;
     // mixed precision: leaf offsets hi|lo (6n floats), float charges and far
     // field, radius-scaled float multipoles for the single-precision M2L
     float *hl = nullptr, *qf = nullptr, *far_phi_f = nullptr, *far_E_f = nullptr;

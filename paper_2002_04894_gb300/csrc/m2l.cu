@@ -20,12 +20,11 @@
 //
 // GPU mapping (double precision): GB300's FP64 pipe retires about two
 // multiply-adds per clock per SM, so the kernel is organised to issue as few
-// FP64 instructions as possible and lets everything else be cheap: one CTA
-// per target box, one weak pair per thread, per-thread coefficient vectors
-// in shared memory (column per thread, conflict-free), D and the axial
-// coefficients in shared memory (every lane reads the same entry: broadcast),
-// and a warp shuffle reduction of the contributions into a per-warp
-// accumulator, so no atomics are needed.
+// FP64 instructions as possible and lets everything else be cheap: one weak
+// pair per thread, per-thread coefficient vectors in shared memory (column per
+// thread, conflict-free), D and the axial coefficients in shared memory (every
+// lane reads the same entry: broadcast), and column sums over the pairs of one
+// target before the atomics.
 
 #include <algorithm>
 #include <cmath>
@@ -42,6 +41,11 @@ namespace fmm {
 
 namespace {
 
+constexpr int kM2LF64Warps = 12;            // warps of a block of the FP64 M2L at most
+constexpr size_t kM2LF64Smem = 227 * 1024;  // its shared memory at most
+constexpr int kM2LF64Unrolled = 12;         // degrees with code of their own
+constexpr int kM2LF64Row = 33;              // pairs' slots between coefficients (32 and one: no bank conflicts)
+
 __device__ __forceinline__ double2 mul_ipow(int m, double2 v) {  // i^m v
     switch (m & 3) {
         case 0: return v;
@@ -51,146 +55,252 @@ __device__ __forceinline__ double2 mul_ipow(int m, double2 v) {  // i^m v
     }
 }
 
-// out_k (k = 0..n) = fold(D^n) applied to v (m = 0..n); transpose: use D_mk.
-__device__ __forceinline__ void fold_apply(const double *__restrict__ D, int n, const double2 *v,
-                                           double2 *out, int stride, bool transpose) {
-    for (int k = 0; k <= n; k++) {
-        double re = 0.0, im = 0.0;
-        const int par = (n + k) & 1;
-        for (int m = par; m <= n; m += 2)
-            re = fma(transpose ? D[m * (n + 1) + k] : D[k * (n + 1) + m], v[m * stride].x, re);
-        for (int m = 1 - par; m <= n; m += 2)
-            im = fma(transpose ? D[m * (n + 1) + k] : D[k * (n + 1) + m], v[m * stride].y, im);
-        out[k * stride] = make_double2(re, im);
+// Folds of degree n in place (v: coefficient (n, 0) of this lane's pair, the
+// next ones kM2LF64Row apart; the m = 0 input and the k = 0 output are real):
+//   v_k = sum_m D_km v_m (kT: D_mk), the results times s0 (k = 0), or sr (real)
+//   and si (imaginary part) with kT.
+// N >= 0: the degree, all of it unrolled and the inputs in registers; N = -1:
+// degree n, the inputs copied to u.
+template <bool kT, int N>
+__device__ __forceinline__ void fold_degree(const double *D, double2 *v, double2 *u, int n, double s0, double sr,
+                                            double si) {
+    constexpr int R = kM2LF64Row;
+    if constexpr (N >= 0) {
+        double2 x[N + 1];
+#pragma unroll
+        for (int m = 0; m <= N; m++) x[m] = v[m * R];
+#pragma unroll
+        for (int k = 0; k <= N; k++) {
+            double re = 0.0, im = 0.0;
+#pragma unroll
+            for (int m = 0; m <= N; m++) {
+                const int i = kT ? m * (N + 1) + k : k * (N + 1) + m;
+                if (((N + k + m) & 1) == 0)
+                    re = fma(D[i], x[m].x, re);
+                else if (m > 0 && k > 0)
+                    im = fma(D[i], x[m].y, im);
+            }
+            if (kT) re *= k ? sr : s0, im *= si;
+            v[k * R] = make_double2(re, im);
+        }
+    } else {
+        for (int m = 0; m <= n; m++) u[m * R] = v[m * R];
+        const int dk = kT ? 1 : n + 1, dm = kT ? n + 1 : 1;
+        for (int k = 0; k <= n; k++, D += dk) {
+            const int par = (n + k) & 1;
+            double re = 0.0, im = 0.0;
+            for (int m = par; m <= n; m += 2) re = fma(D[m * dm], u[m * R].x, re);
+            for (int m = par ? 2 : 1; m <= n && k > 0; m += 2) im = fma(D[m * dm], u[m * R].y, im);
+            if (kT) re *= k ? sr : s0, im *= si;
+            v[k * R] = make_double2(re, im);
+        }
     }
 }
 
+// The axial translation of one order l in place: the len = p + 1 - l
+// coefficients of degrees l..p, `l` + 1, `l` + 2, .. slots apart.
+template <int LEN>
+__device__ __forceinline__ void axial_order(const double *A, double2 *v, double2 *u, int l, int len) {
+    constexpr int R = kM2LF64Row;
+    if constexpr (LEN > 0) {
+        double2 x[LEN];
+#pragma unroll
+        for (int j = 0; j < LEN; j++) x[j] = v[(j * l + j * (j + 1) / 2) * R];
+#pragma unroll
+        for (int k = 0; k < LEN; k++) {
+            double re = 0.0, im = 0.0;
+#pragma unroll
+            for (int j = 0; j < LEN; j++) {
+                re = fma(A[k * LEN + j], x[j].x, re);
+                im = fma(A[k * LEN + j], x[j].y, im);
+            }
+            v[(k * l + k * (k + 1) / 2) * R] = make_double2(re, im);
+        }
+    } else {
+        for (int j = 0; j < len; j++) u[j * R] = v[(j * l + j * (j + 1) / 2) * R];
+        for (int k = 0; k < len; k++, A += len) {
+            double re = 0.0, im = 0.0;
+            for (int j = 0; j < len; j++) {
+                re = fma(A[j], u[j * R].x, re);
+                im = fma(A[j], u[j * R].y, im);
+            }
+            v[(k * l + k * (k + 1) / 2) * R] = make_double2(re, im);
+        }
+    }
+}
+
+extern __shared__ double2 m2l64_sm[];
+
+#define FMM_M2L64_CASES(X) X(0) X(1) X(2) X(3) X(4) X(5) X(6) X(7) X(8) X(9) X(10) X(11) X(12)
+
+// All degrees; results of degree n times s ratio^n, wr and wi more for k > 0 (kT).
+template <bool kT>
+__device__ __noinline__ void fold_degrees(int p, int slot, int spare, double s, double ratio, double wr, double wi) {
+    const double *D = (const double *)m2l64_sm;
+    double2 *v = m2l64_sm + slot, *u = m2l64_sm + spare;
+    for (int n = 0; n <= p; n++) {
+        const double sr = wr * s, si = wi * s;
+        switch (n) {
+#define FMM_X(N) \
+    case N: fold_degree<kT, N>(D, v, u, N, s, sr, si); break;
+            FMM_M2L64_CASES(FMM_X)
+#undef FMM_X
+            default: fold_degree<kT, -1>(D, v, u, n, s, sr, si);
+        }
+        D += (n + 1) * (n + 1);
+        v += (n + 1) * kM2LF64Row;
+        s *= ratio;
+    }
+}
+
+__device__ __noinline__ void axial_orders(int p, int slot, int spare, int tab) {
+    const double *A = (const double *)m2l64_sm + tab;
+    double2 *v = m2l64_sm + slot, *u = m2l64_sm + spare;
+    for (int l = 0; l <= p; l++) {
+        const int len = p + 1 - l;
+        switch (len - 1) {
+#define FMM_X(N) \
+    case N: axial_order<N + 1>(A, v, u, l, len); break;
+            FMM_M2L64_CASES(FMM_X)
+#undef FMM_X
+            default: axial_order<0>(A, v, u, l, len);
+        }
+        A += len * len;
+        v += (l + 2) * kM2LF64Row;  // from (l, l) to (l + 1, l + 1)
+    }
+}
+#undef FMM_M2L64_CASES
+
+// v_{n,m} *= w s^m for every degree n and order m > 0 (w: 1 or 2, exact).
+__device__ __noinline__ void phase_orders(int p, int slot, double w, double2 s) {
+    double2 ph = make_double2(w * s.x, w * s.y);
+    double2 *col = m2l64_sm + slot + 2 * kM2LF64Row;  // (m, m)
+    for (int m = 1; m <= p; m++) {
+        double2 *x = col;
+        int n = m;
+        for (; n + 1 <= p; n += 2) {
+            double2 *y = x + (n + 1) * kM2LF64Row;
+            const double2 a = *x, b = *y;
+            *x = cmul(a, ph);
+            *y = cmul(b, ph);
+            x = y + (n + 2) * kM2LF64Row;
+        }
+        if (n == p) *x = cmul(*x, ph);
+        col += (m + 2) * kM2LF64Row;
+        ph = cmul(ph, s);
+    }
+}
+
+// One weak pair per lane, 32 pairs of (mostly) one target per warp; warps
+// stride over the pairs by themselves, a few of them per SM (their vectors fill
+// the shared memory: 35 KB a warp at p = 10), one block per SM.
+//
+// Few FP64 operations, and code that keeps the pipe (one warp instruction per
+// ~19 cycles and SM) fed from six warps at p = 10: the powers of the phases are
+// formed once per pair (the phase steps run order by order over all degrees),
+// the factors rho^-n ride on the folds' results, the powers of i cancel across
+// the translation (i^l conj(i^l z) = conj z) or join the azimuthal phase, zero
+// imaginary parts take no part, and a warp's results are summed by columns in
+// shared memory (one addition per pair and value, not five shuffled ones), F_nm
+// applied to the sums: about 3,900 operations per pair at p = 10 where phases
+// per degree and shuffled sums took 6,930. The folds and the translation are
+// unrolled per degree with their inputs in registers: as loops a warp issued an
+// FP64 instruction every ~113 cycles however many sums ran side by side. Time,
+// before -> now: 1.03e6 pairs at p = 10 16.9 -> 8.8 ms, 1.65e7 270 -> 141 ms
+// (67% of the measured FP64 peak by the contractions' plain count), 13,254
+// pairs 0.215 -> 0.127 ms. Few pairs or many, it is the FP64 pipe that bounds it
+// (~23 cycles per instruction and SM).
+//
 // With ext_M set, the sources are not boxes of the plan: pair g is (target
 // box PT.tgt[PT.lmin][g] of level PT.lmin, source g with multipole ext_M[g]
 // about ext_centre[g]) -- a split system's multipoles from another rank; the
-// targets are then in no particular order, so each pair adds its own result.
-__global__ void k_m2l_rot_f64(PairTable PT, int p, const double *__restrict__ centre,
-                              const double2 *__restrict__ M, double2 *__restrict__ L,
-                              const double *__restrict__ gtab, int ntab,
-                              const double *__restrict__ ext_centre = nullptr,
-                              const double2 *__restrict__ ext_M = nullptr) {
-    extern __shared__ double2 sm2[];
-    const int nc = ncoef(p), T = blockDim.x, tid = threadIdx.x;
-    // shared layout: [V: nc*T][U: (p+1)*T][W: (p+1)*T][tables: ntab doubles]
-    double2 *V = sm2;
-    double2 *U = V + nc * T;
-    double2 *W = U + (p + 1) * T;
-    double *tab = (double *)(W + (p + 1) * T);
-    for (int i = tid; i < ntab; i += T) tab[i] = gtab[i];
+// targets are then in no particular order (neighbours that happen to be equal
+// are summed like any run).
+__global__ void __launch_bounds__(kM2LF64Warps * 32)
+k_m2l_rot_f64(PairTable PT, int p, const double *__restrict__ centre,
+              const double2 *__restrict__ M, double2 *__restrict__ L,
+              const double *__restrict__ gtab, int ntab,
+              const double *__restrict__ ext_centre, const double2 *__restrict__ ext_M) {
+    constexpr int R = kM2LF64Row;
+    const int nc = ncoef(p), lane = threadIdx.x & 31, warp = threadIdx.x >> 5, W = blockDim.x >> 5;
+    // shared layout: [tables: ntab doubles][per warp: nc * R, and (p + 1) * R for long degrees]
+    double *tab = (double *)m2l64_sm;
+    for (int i = threadIdx.x; i < ntab; i += blockDim.x) tab[i] = gtab[i];
     __syncthreads();
     // tables: D (sum (n+1)^2), axial A (sum_l (p+1-l)^2), F_nm (nc)
-    const double *Dt = tab;
     const int nD = (p + 1) * (p + 2) * (2 * p + 3) / 6;
-    const double *At = Dt + nD;
-    const double *Ft = At + nD;
-    double2 *v = V + tid, *u = U + tid, *x = W + tid;
-
-    const int64_t g = blockIdx.x * (int64_t)T + tid;
-    const bool valid = g < PT.off[PT.lmax + 1];
-    int64_t gt = -1, gs = 0;
-    double dx = 1.0, dy = 0.0, dz = 0.0;
+    const double *Ft = tab + 2 * nD;
+    const int base = (ntab + 1) / 2 + warp * R * (nc + (p > kM2LF64Unrolled ? p + 1 : 0));
+    const int slot = base + lane, spare = slot + nc * R;
+    double2 *v = m2l64_sm + slot;
     const double *cs = ext_M ? ext_centre : centre;
     const double2 *Ms = ext_M ? ext_M : M;
-    if (valid) {
-        if (ext_M) {
-            gt = ((int64_t)1 << PT.lmin) - 1 + PT.tgt[PT.lmin][g];
-            gs = g;
-        } else {
-            pair_of(PT, g, gt, gs);
-        }
-        dx = centre[3 * gt] - cs[3 * gs];
-        dy = centre[3 * gt + 1] - cs[3 * gs + 1];
-        dz = centre[3 * gt + 2] - cs[3 * gs + 2];
-    }
-    bool same[5], head;
-    seg_setup(gt, same, head);
-    if (ext_M) {  // external pairs come in any order: no run sums, one atomic add per pair
-#pragma unroll
-        for (int j = 0; j < 5; j++) same[j] = false;
-        head = valid;
-    }
-    const double rxy = sqrt(dx * dx + dy * dy);
-    const double rho = sqrt(dx * dx + dy * dy + dz * dz);
-    const double rinv = 1.0 / rho;
-    const double2 ea = rxy > 0.0 ? make_double2(dx / rxy, dy / rxy) : make_double2(1.0, 0.0);
-    const double2 eb_ = make_double2(dz * rinv, rxy * rinv);
-    const double2 eai = make_double2(ea.y, -ea.x);  // -i e^{ia}
+    const int64_t total = PT.off[PT.lmax + 1];
 
-    // ---- forward rotation, degree by degree -> v = Mr (F-normalised)
-    const double *Dn = Dt;
-    for (int n = 0; n <= p; n++) {
-        double2 ph = make_double2(1.0, 0.0);
-        for (int m = 0; m <= n; m++) {
-            const int c = tri(n, m);
-            const double2 mv = valid ? Ms[gs * nc + c] : make_double2(0.0, 0.0);
-            u[m * T] = cscale(cmul(mv, ph), Ft[c] * (m ? 2.0 : 1.0));
-            ph = cmul(ph, eai);
-        }
-        fold_apply(Dn, n, u, x, T, false);
-        double2 pb = make_double2(1.0, 0.0);
-        for (int k = 0; k <= n; k++) {
-            x[k * T] = cscale(cmul(x[k * T], pb), k ? 2.0 : 1.0);
-            pb = cmul(pb, eb_);
-        }
-        fold_apply(Dn, n, x, u, T, true);
-        for (int m = 0; m <= n; m++) v[tri(n, m) * T] = mul_ipow(m, u[m * T]);
-        Dn += (n + 1) * (n + 1);
-    }
-    // ---- translation along z, order by order (in place)
-    const double *Al = At;
-    double rl = 1.0;  // rho^-l
-    for (int l = 0; l <= p; l++) {
-        const int len = p + 1 - l;
-        double rp = rl;
-        for (int n = l; n <= p; n++) {
-            const double2 mr = v[tri(n, l) * T];
-            u[(n - l) * T] = make_double2(mr.x * rp, -mr.y * rp);
-            rp *= rinv;
-        }
-        double rk = rl * rinv;  // rho^-(k+1) at k = l
-        for (int k = l; k <= p; k++) {
-            double re = 0.0, im = 0.0;
-            const double *a = Al + (k - l) * len;
-            for (int j = 0; j < len; j++) {
-                const double2 s = u[j * T];
-                re = fma(a[j], s.x, re);
-                im = fma(a[j], s.y, im);
+    for (int64_t g0 = ((int64_t)blockIdx.x * W + warp) * 32; g0 < total; g0 += (int64_t)gridDim.x * W * 32) {
+        const int64_t g = g0 + lane;
+        const bool valid = g < total;
+        int64_t gt = -1, gs = 0;
+        double dx = 1.0, dy = 0.0, dz = 0.0;
+        if (valid) {
+            if (ext_M) {
+                gt = ((int64_t)1 << PT.lmin) - 1 + PT.tgt[PT.lmin][g];
+                gs = g;
+            } else {
+                pair_of(PT, g, gt, gs);
             }
-            v[tri(k, l) * T] = make_double2(re * rk, im * rk);
-            rk *= rinv;
+            dx = centre[3 * gt] - cs[3 * gs];
+            dy = centre[3 * gt + 1] - cs[3 * gs + 1];
+            dz = centre[3 * gt + 2] - cs[3 * gs + 2];
         }
-        Al += len * len;
-        rl *= rinv;
-    }
-    // ---- inverse rotation, degree by degree; segmented reduction per target
-    Dn = Dt;
-    for (int k = 0; k <= p; k++) {
-        for (int m = 0; m <= k; m++)
-            u[m * T] = cscale(mul_ipow(m, v[tri(k, m) * T]), m ? 2.0 : 1.0);
-        fold_apply(Dn, k, u, x, T, false);
-        double2 pb = make_double2(1.0, 0.0);
-        for (int j = 0; j <= k; j++) {
-            x[j * T] = cscale(cmul(x[j * T], pb), j ? 2.0 : 1.0);
-            pb = cmul(pb, eb_);
-        }
-        fold_apply(Dn, k, x, u, T, true);
-        double2 ph = make_double2(1.0, 0.0);
-        for (int l = 0; l <= k; l++) {
-            const int c = tri(k, l);
-            const double2 r = cscale(cmul(mul_ipow(4 - (l & 3), u[l * T]), ph), Ft[c]);
-            const double rx = seg_sum(r.x, same), ry = seg_sum(r.y, same);
-            if (head) {
-                atomicAdd(&L[gt * nc + c].x, rx);
-                atomicAdd(&L[gt * nc + c].y, ry);
+        const double rxy = sqrt(dx * dx + dy * dy);
+        const double rho = sqrt(dx * dx + dy * dy + dz * dz);
+        const double rinv = 1.0 / rho;
+        const double2 ea = rxy > 0.0 ? make_double2(dx / rxy, dy / rxy) : make_double2(1.0, 0.0);
+        const double2 eb = make_double2(dz * rinv, rxy * rinv);
+        const double2 eai = make_double2(ea.y, -ea.x);  // -i e^{ia}
+        const double2 *row = Ms + gs * nc;
+#pragma unroll 8
+        for (int c = 0; c < nc; c++) v[c * R] = valid ? cscale(row[c], Ft[c]) : make_double2(0.0, 0.0);
+        // forward rotation; its results rho^-n conj(Mr), doubled for m > 0 for the next fold
+        phase_orders(p, slot, 2.0, eai);
+        fold_degrees<false>(p, slot, spare, 1.0, 1.0, 1.0, 1.0);
+        phase_orders(p, slot, 2.0, eb);
+        fold_degrees<true>(p, slot, spare, 1.0, rinv, 2.0, -2.0);
+        axial_orders(p, slot, spare, nD);
+        // inverse rotation, times rho^-(k+1)
+        fold_degrees<false>(p, slot, spare, 1.0, 1.0, 1.0, 1.0);
+        phase_orders(p, slot, 2.0, eb);
+        fold_degrees<true>(p, slot, spare, rinv, rinv, 1.0, 1.0);
+        phase_orders(p, slot, 1.0, eai);
+        // sums over the runs of equal targets: one lane per value, row by row
+        __syncwarp();
+        const int nv = __popc(__ballot_sync(0xffffffffu, valid));
+        const int64_t next = __shfl_down_sync(0xffffffffu, gt, 1);
+        const unsigned ends = __ballot_sync(0xffffffffu, valid && (lane + 1 == nv || next != gt));
+        for (int c0 = 0; c0 < 2 * nc; c0 += 128) {  // four values a lane at a time
+            const double *col[4];
+            double s[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+            for (int j = 0; j < 4; j++) {
+                const int d = min(c0 + 32 * j + lane, 2 * nc - 1);
+                col[j] = (const double *)(m2l64_sm + base + (d >> 1) * R) + (d & 1);
             }
-            ph = cmul(ph, ea);
+            for (int i = 0; i < nv; i++) {
+#pragma unroll
+                for (int j = 0; j < 4; j++) s[j] += col[j][2 * i];
+                if (ends >> i & 1) {
+                    const int64_t t = __shfl_sync(0xffffffffu, gt, i);
+#pragma unroll
+                    for (int j = 0; j < 4; j++) {
+                        const int d = c0 + 32 * j + lane;
+                        if (d < 2 * nc) atomicAdd((double *)(L + t * nc) + d, s[j] * Ft[d >> 1]);
+                        s[j] = 0.0;
+                    }
+                }
+            }
         }
-        Dn += (k + 1) * (k + 1);
+        __syncwarp();
     }
 }
 
@@ -1114,6 +1224,28 @@ const std::vector<double> &m2l_tables_cached(int p) {
     return cache[p];
 }
 
+// Shared memory of a block of W warps of the FP64 M2L, and the warps of order p:
+// as many as fit (p = 8: 9, p = 10: 6, p = 12: 4, p = 20: 1).
+static size_t m2l_f64_smem(int p, int W, int ntab) {
+    const size_t slots = ncoef(p) + (p > kM2LF64Unrolled ? p + 1 : 0);
+    return ((size_t)(ntab + 1) / 2 + W * slots * kM2LF64Row) * 16;
+}
+static int m2l_f64_warps(int p, int ntab) {
+    int W = 1;
+    while (W < kM2LF64Warps && m2l_f64_smem(p, W + 1, ntab) <= kM2LF64Smem) W++;
+    return W;
+}
+// Few pairs: only as many warps as give every SM its share (13,254 pairs at
+// p = 10: 139 blocks of three warps).
+static void m2l_f64_launch(Plan &P, const PairTable &PT, int64_t n, const double2 *M, double2 *L,
+                           const double *ext_centre, const double2 *ext_M) {
+    const int64_t chunks = (n + 31) / 32, sms = sm_count();
+    const int W = (int)std::min<int64_t>(P.m2l_warps, (chunks + sms - 1) / sms);
+    const unsigned grid = (unsigned)std::min<int64_t>(sms, (chunks + W - 1) / W);
+    FMM_LAUNCH(k_m2l_rot_f64, grid, W * 32, m2l_f64_smem(P.p, W, P.m2l_ntab), P.stream, PT, P.p, P.centre, M, L,
+               P.m2l_tab, P.m2l_ntab, ext_centre, ext_M);
+}
+
 cudaError_t m2l_setup(Plan &P) {
     const std::vector<double> &both = m2l_tables_cached(P.p);
     const size_t nt = both.size() / 2, up = P.prec == FMM_PREC_MIXED ? 2 * nt : nt;
@@ -1134,13 +1266,8 @@ cudaError_t m2l_setup(Plan &P) {
         FMM_LAUNCH(k_box_geo, (unsigned)std::min<int64_t>((P.nbox + 255) / 256, (int64_t)sm_count() * 8), 256, 0,
                    P.stream, P.nbox, P.step, P.centre, P.radius, (BoxGeo *)P.box_geo);
     }
-    const int nc = P.nc;
-    int threads = 64;
-    auto smem = [&](int T) { return (size_t)T * (nc + 2 * (P.p + 1)) * 16 + nt * 8; };
-    if (smem(threads) > 220 * 1024) threads = 32;
-    P.m2l_threads = threads;
-    P.m2l_smem = smem(threads);
-    e = allow_max_smem((const void *)k_m2l_rot_f64, P.m2l_smem);
+    P.m2l_warps = m2l_f64_warps(P.p, (int)nt);
+    e = allow_max_smem((const void *)k_m2l_rot_f64, m2l_f64_smem(P.p, P.m2l_warps, (int)nt));
     const size_t grp_max = (size_t)kWarpChildMax * warp_slice(P.p) * 16 + (size_t)warp_tabs(P.p) * 8;
     const void *kernels[] = {(const void *)k_l2l_warp<false>, (const void *)k_m2m_warp<false>,
                              (const void *)k_m2m_up<false>,   (const void *)k_l2l_down<false>,
@@ -1200,8 +1327,7 @@ cudaError_t m2l_external(Plan &P, int level, int64_t n, const int32_t *tgt, cons
     PT.tgt[level] = tgt;
     PT.off[level] = 0;
     PT.off[level + 1] = n;
-    FMM_LAUNCH(k_m2l_rot_f64, (unsigned)((n + P.m2l_threads - 1) / P.m2l_threads), P.m2l_threads, P.m2l_smem,
-               P.stream, PT, P.p, P.centre, (const double2 *)nullptr, P.L_ext, P.m2l_tab, P.m2l_ntab, csrc, Msrc);
+    m2l_f64_launch(P, PT, n, nullptr, P.L_ext, csrc, Msrc);
     return cudaGetLastError();
 }
 
@@ -1255,8 +1381,7 @@ cudaError_t m2l_all(Plan &P) {
     cudaMemsetAsync(P.L, 0, (size_t)P.nbox * P.nc * sizeof(double2), P.stream);
     const int64_t tot = total_weak(P);
     if (tot == 0) return cudaGetLastError();
-    FMM_LAUNCH(k_m2l_rot_f64, (unsigned)((tot + P.m2l_threads - 1) / P.m2l_threads), P.m2l_threads,
-               P.m2l_smem, P.stream, pair_table(P), P.p, P.centre, P.M, P.L, P.m2l_tab, P.m2l_ntab);
+    m2l_f64_launch(P, pair_table(P), tot, P.M, P.L, nullptr, nullptr);
     return cudaGetLastError();
 }
 
