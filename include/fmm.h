@@ -53,8 +53,9 @@ enum fmm_status {
     FMM_ENOMEM = -2,      /* the allocator returned NULL */
     FMM_ENONFINITE = -3,  /* a point coordinate is NaN or infinite */
     FMM_ECAPACITY = -4,   /* an interaction list exceeds 2^31 - 1 entries */
-    FMM_ETIMEDOUT = -5,   /* a bounded device wait gave up (one-launch downward pass,
-                             tensor-core M2L); reported by fmm_eval_check */
+    FMM_ETIMEDOUT = -5,   /* a bounded device wait gave up (one-launch downward pass, copies of
+                             the mixed form's M2L, tensor-core M2L); reported by
+                             fmm_eval_check */
     FMM_ECUDA = -6,       /* a CUDA runtime call failed; fmm_last_cuda_error() has the code */
     FMM_EINTERNAL = -7    /* a device-side consistency check of the tree build failed (the
                              partition of a box did not give the sizes the split rule

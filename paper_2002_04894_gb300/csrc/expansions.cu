@@ -80,7 +80,7 @@ __device__ __forceinline__ void harmonics(int p, double v0, double x, double y, 
 // terms of eight coefficients at a time go to shared memory and are summed by
 // columns, two lanes to a column (about 2 operations per point and coefficient
 // where a shuffled sum takes 10), the charge and the signs ride on the
-// recurrence. 200,000 points at p = 10: 0.96 -> 0.34 ms, 20,000 points 78 -> 35 us.
+// recurrence. 200,000 points at p = 10: 0.96 -> 0.34 ms, 20,000 at p = 8 78 -> 35 us.
 constexpr int kP2MCols = 16;  // real columns of a batch of sums (two lanes to a column of 32 terms)
 __global__ void __launch_bounds__(kExpThreads)
 k_p2m(int B, int p, const double *__restrict__ x, const double *__restrict__ y,
@@ -138,7 +138,7 @@ k_p2m(int B, int p, const double *__restrict__ x, const double *__restrict__ y,
 //   g1 += L_n+1,m+1 conj Y - conj(L_n+1,m-1) Y
 // The factors are combined per leaf first (Ls: four pairs per coefficient), so
 // a point takes eight multiply-adds a coefficient beside the recurrence's
-// seven. 200,000 points at p = 10: 1.00 -> 0.44 ms, 20,000 points 76 -> 41 us.
+// seven. 200,000 points at p = 10: 1.00 -> 0.44 ms, 20,000 at p = 8 76 -> 41 us.
 __global__ void __launch_bounds__(kExpThreads)
 k_l2p(int B, int p, int64_t npts, const double *__restrict__ x, const double *__restrict__ y,
       const double *__restrict__ z, const int32_t *__restrict__ begin,

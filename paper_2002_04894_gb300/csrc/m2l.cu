@@ -208,7 +208,7 @@ __device__ __noinline__ void phase_orders(int p, int slot, double w, double2 s) 
 // FP64 instruction every ~113 cycles however many sums ran side by side. Time,
 // before -> now: 1.03e6 pairs at p = 10 16.9 -> 8.8 ms, 1.65e7 270 -> 141 ms
 // (67% of the measured FP64 peak by the contractions' plain count), 13,254
-// pairs 0.215 -> 0.127 ms. Few pairs or many, it is the FP64 pipe that bounds it
+// pairs at p = 8 0.215 -> 0.127 ms. Few pairs or many, it is the FP64 pipe that bounds it
 // (~23 cycles per instruction and SM).
 //
 // With ext_M set, the sources are not boxes of the plan: pair g is (target
@@ -1235,8 +1235,8 @@ static int m2l_f64_warps(int p, int ntab) {
     while (W < kM2LF64Warps && m2l_f64_smem(p, W + 1, ntab) <= kM2LF64Smem) W++;
     return W;
 }
-// Few pairs: only as many warps as give every SM its share (13,254 pairs at
-// p = 10: 139 blocks of three warps).
+// Few pairs: only as many warps as give every SM its share (13,254 pairs:
+// 139 blocks of three warps).
 static void m2l_f64_launch(Plan &P, const PairTable &PT, int64_t n, const double2 *M, double2 *L,
                            const double *ext_centre, const double2 *ext_M) {
     const int64_t chunks = (n + 31) / 32, sms = sm_count();
