@@ -1,13 +1,14 @@
 // Near field of the FP64 form (P2P, Algorithm 4) in three-float arithmetic.
 //
-// What bounds it: the FP32 pipe (84% busy). A pair takes ~360 packed
+// What bounds it: the FP32 pipe. A pair takes ~295 packed
 // operations (trifloat.cuh) where FP64 arithmetic takes 19 FP64 instructions at
 // less than two per clock and SM, ~1,400 FP32 operations' time, and its terms
 // are more accurate than those of plain double arithmetic. Sums run in
-// TwoSum-compensated three-float accumulators. 200k Plummer points, 11 levels,
-// 1.16e10 pairs: FP64 arithmetic 412.6 ms (its pipe saturated), this 124.5;
-// 20k uniform points, 8 levels: 3.29 -> 1.05 ms. Registers: 4 blocks of 128
-// threads per SM (128 registers; 5 blocks 127.9 ms, 6 132.7). With block-wide
+// compensated three-float accumulators. 200k Plummer points, 11 levels,
+// 1.16e10 pairs: FP64 arithmetic 412.6 ms (its pipe saturated), this 110.7;
+// 20k uniform points, 8 levels: 3.29 -> 0.95 ms. Registers: 4 blocks of 128
+// threads per SM (128 registers; with ~365 operations a pair 124.5 ms, 5 blocks
+// 127.9, 6 132.7). With block-wide
 // staging and its barriers: 152.9 ms.
 //
 // Positions are taken relative to the root cell's centre on a common grid of
@@ -105,24 +106,25 @@ __device__ __forceinline__ float charge_split(double q, int e, float thr, float 
 
 __device__ __forceinline__ void clear_x(tf::PairTerms<float2> &o) {
     o.phi.a.x = o.phi.b.x = o.phi.c.x = 0.f;
-#pragma unroll
-    for (int a = 0; a < 3; a++) o.e[a].a.x = o.e[a].b.x = o.e[a].c.x = 0.f;
+    o.w.a.x = o.w.b.x = o.w.c.x = 0.f;
 }
 __device__ __forceinline__ void clear_y(tf::PairTerms<float2> &o) {
     o.phi.a.y = o.phi.b.y = o.phi.c.y = 0.f;
-#pragma unroll
-    for (int a = 0; a < 3; a++) o.e[a].a.y = o.e[a].b.y = o.e[a].c.y = 0.f;
+    o.w.a.y = o.w.b.y = o.w.c.y = 0.f;
 }
 
 // the sums of positions over 2^k and charges over 2^eq, and the FP64 pairs
-__device__ __forceinline__ double4 result(const tf::Acc<float2> (&A)[4], const double (&slow)[4], int k, int eq) {
-    double v[4];
+template <bool F>
+__device__ __forceinline__ double4 result(const tf::Sums<float2, F> &A, const double (&slow)[4], int k, int eq) {
+    double v[4] = {slow[0], slow[1], slow[2], slow[3]};
 #pragma unroll
-    for (int c = 0; c < 4; c++)
-        v[c] = scalbn(((double)A[c].a.x + (double)A[c].a.y) +
-                          (((double)A[c].b.x + (double)A[c].b.y) + ((double)A[c].c.x + (double)A[c].c.y)),
-                      c ? eq - 2 * k : eq - k) +
-               slow[c];
+    for (int c = 0; c < tf::Sums<float2, F>::N; c++) {
+        const double m = A.M[c > 0];
+        v[c] += scalbn(((double)A.a[c].x + (double)A.a[c].y) +
+                           ((((double)A.s[c].x - m) + ((double)A.s[c].y - m)) +
+                            ((double)A.c[c].x + (double)A.c[c].y)),
+                       c ? eq - 2 * k : eq - k);
+    }
     return make_double4(v[0], v[1], v[2], v[3]);
 }
 
@@ -193,8 +195,7 @@ k_p2p_tf(int B, int64_t n, const double *__restrict__ x, const double *__restric
         X[a] = {make_float2(f[0], f[0]), make_float2(f[1], f[1]), make_float2(f[2], f[2])};
     }
     if (L.active) thr_i = thr0[slot];
-    const float2 zero = make_float2(0.f, 0.f);
-    tf::Acc<float2> A[4] = {{zero, zero, zero}, {zero, zero, zero}, {zero, zero, zero}, {zero, zero, zero}};
+    tf::Sums<float2, F> A(make_float2(0.f, 0.f));
     double slow[4] = {0.0, 0.0, 0.0, 0.0};
     float4(*sm)[kChunk / 2] = sm_all[tid >> 5];
     float2 *sthr = sthr_all[tid >> 5];
@@ -250,10 +251,10 @@ k_p2p_tf(int B, int64_t n, const double *__restrict__ x, const double *__restric
                         clear_y(o);
                     }
                 }
-                A[0].put(o.phi);
-#pragma unroll
-                for (int a = 0; a < (F ? 3 : 0); a++) A[1 + a].put(o.e[a]);
+                A.put_phi(o.phi);
+                if constexpr (F) A.put_field(o.w, o.d);
             }
+            A.settle();
         }
     }
     int k;
@@ -281,7 +282,7 @@ k_p2p_tf(int B, int64_t n, const double *__restrict__ x, const double *__restric
 // slab and adds its sums to the (segment, target) slot; a last pass adds the
 // segments. 500k points, 1000 targets (5e8 pairs): one block per target in FP64
 // arithmetic (square root, two divisions and Neumaier sums a pair) 58.6 ms,
-// this 5.48 (85% of the FP32 pipe's rate for ~377 operations a pair); 1 target:
+// this 4.92 (~295 operations a pair; ~365: 5.48); 1 target:
 // 8.40 -> 0.36 ms, 2000 points and 1000 targets 0.38 -> 0.08.
 // ---------------------------------------------------------------------------
 constexpr int kRec = 7;
@@ -430,12 +431,11 @@ k_direct_tf(const T *__restrict__ pts, const T *__restrict__ q, int64_t n, const
 #pragma unroll
     for (int a = 0; a < 3; a++)
         X[a] = {make_float2(f[a][0], f[a][0]), make_float2(f[a][1], f[a][1]), make_float2(f[a][2], f[a][2])};
-    const float2 zero = make_float2(0.f, 0.f);
-    tf::Acc<float2> A[4] = {{zero, zero, zero}, {zero, zero, zero}, {zero, zero, zero}, {zero, zero, zero}};
+    tf::Sums<float2, true> A(make_float2(0.f, 0.f));
     double slow[4] = {0.0, 0.0, 0.0, 0.0};
     const int64_t np = (j1 - j0 + 1) >> 1, p1 = busy ? min(np, (blockIdx.y + 1) * len) : 0;
 #pragma unroll 1
-    for (int64_t pp = blockIdx.y * len + L.slice; pp < p1; pp += L.slices) {
+    for (int64_t pp = blockIdx.y * len + L.slice, terms = 1; pp < p1; pp += L.slices, terms++) {
         const float4 *r = rec + pp * kRec;
         const float4 a0 = __ldg(r), a1 = __ldg(r + 1), b0 = __ldg(r + 2), b1 = __ldg(r + 3), c0 = __ldg(r + 4),
                      c1 = __ldg(r + 5), th = __ldg(r + 6);
@@ -456,10 +456,11 @@ k_direct_tf(const T *__restrict__ pts, const T *__restrict__ q, int64_t n, const
                 clear_y(o);
             }
         }
-        A[0].put(o.phi);
-#pragma unroll
-        for (int a = 0; a < 3; a++) A[1 + a].put(o.e[a]);
+        A.put_phi(o.phi);
+        A.put_field(o.w, o.d);
+        if ((terms & 31) == 0) A.settle();
     }
+    A.settle();
     double4 r = result(A, slow, box->grid.k, box->grid.eq);
     if (L.combine(r, red)) {
         double4 *slot = partial + blockIdx.y * nt + t0 + L.target;

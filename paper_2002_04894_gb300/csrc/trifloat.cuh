@@ -2,13 +2,14 @@
 //
 // GB300 retires 128 FP32 operations per clock and SM, but fewer than two FP64
 // ones, so an FP64 pair (19 FP64 instructions) costs as much as ~1,400 FP32
-// operations. Here a pair takes about 360: every quantity is an unevaluated
+// operations. Here a pair takes about 295: every quantity is an unevaluated
 // sum of three floats (~72 bits), built from error-free transformations
 // (Knuth's TwoSum, Dekker's FastTwoSum, the product's rounding error from the
 // fused multiply-add). Terms of the same size are summed exactly by a
 // FastTwoSum chain that starts from a constant M larger than all of them; M
 // comes off exactly at the end. Every operation is an explicitly rounded
-// intrinsic on packed pairs (two sources at once).
+// intrinsic on packed pairs (two sources at once); signs are flipped on the
+// ALU pipe.
 //
 // A pair whose positions are exact on the common grid has relative errors of
 // at most 2^-61 (potential) and 2^-58 (field) over 1.6 million random pairs at
@@ -35,6 +36,11 @@ __device__ __forceinline__ float rsqrt1(float x) {
     asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
+// by the sign bits: the ALU pipe has room, the FMA pipe has none
+__device__ __forceinline__ float2 neg(float2 a) {
+    return make_float2(__int_as_float(__float_as_int(a.x) ^ 0x80000000), __int_as_float(__float_as_int(a.y) ^ 0x80000000));
+}
+__device__ __forceinline__ float amax(float2 x) { return fmaxf(fabsf(x.x), fabsf(x.y)); }
 __device__ __forceinline__ float2 rsqrt0(float2 x) { return make_float2(rsqrt1(x.x), rsqrt1(x.y)); }
 #define TF_DEV __device__ __forceinline__
 #else
@@ -43,6 +49,8 @@ inline float mul(float a, float b) { return a * b; }
 inline float fma(float a, float b, float c) { return fmaf(a, b, c); }
 inline float sub(float a, float b) { return a - b; }
 inline float cst(float, float c) { return c; }
+inline float neg(float a) { return -a; }
+inline float amax(float x) { return fabsf(x); }
 inline float rsqrt0(float x) { return 1.f / sqrtf(x) * TF_RSQRT_ERR; }
 #define TF_DEV inline
 #endif
@@ -52,8 +60,6 @@ struct Tri {
     V a, b, c;  // a + b + c
 };
 
-template <class V>
-TF_DEV V neg(V a) { return mul(a, cst(a, -1.f)); }
 // (By a compare and selects on the ALU pipe and a FastTwoSum instead: the near
 // field of 200k points took 128.2 ms against 124.5.)
 template <class V>
@@ -113,31 +119,21 @@ TF_DEV Tri<V> product(const Tri<V> &A, V nA, V nAb, const Tri<V> &B, V p, V M) {
     return {p, S.top(), t};
 }
 
-// running sum of three-float terms: TwoSums on the first two parts
-template <class V>
-struct Acc {
-    V a, b, c;
-    TF_DEV void put(const Tri<V> &x) {
-        V e1, e2, e3;
-        a = two_sum(a, x.a, e1);
-        b = two_sum(b, x.b, e2);
-        b = two_sum(b, e1, e3);
-        c = add(c, add(add(e2, e3), x.c));
-    }
-};
-
-// One pair (two in packed form): the squared distance's leading part, q / r
-// and q d / r^3 for target x, source y (coordinates negated) and its charge.
+// One pair (two in packed form) for target x, source y (coordinates negated)
+// and its charge: the squared distance's leading part, q / r, W = q / r^3 and
+// d = x - y (the field is W d).
 template <class V>
 struct PairTerms {
     V r2;  // leading part of the squared distance
-    Tri<V> phi, e[3];
+    Tri<V> phi, w, d[3];
 };
 
 template <class V, bool F = true>  // F: with the field
 TF_DEV PairTerms<V> pair_terms(const Tri<V> (&x)[3], const Tri<V> (&ny)[3], const Tri<V> &q) {
     PairTerms<V> o;
-    const Tri<V> d[3] = {diff(x[0], ny[0]), diff(x[1], ny[1]), diff(x[2], ny[2])};
+    const Tri<V> (&d)[3] = o.d;
+#pragma unroll
+    for (int i = 0; i < 3; i++) o.d[i] = diff(x[i], ny[i]);
     const V nh[3] = {neg(d[0].a), neg(d[1].a), neg(d[2].a)};
     // r2 = P + R2 + R3
     V P, R2, R3;
@@ -170,26 +166,29 @@ TF_DEV PairTerms<V> pair_terms(const Tri<V> (&x)[3], const Tri<V> (&ny)[3], cons
         R3 = fma(tau, cst(tau, 2.f), t);
     }
     o.r2 = P;
-    // 1 / r = Y: a Newton-like step on the hardware's y0 with the residual
-    // e = 1 - r2 y0^2 exact to ~2^-54: y0 (1 + e / 2 + 3 e^2 / 8)
+    // The hardware's y0 ~ 1 / r and z, y0^2 rounded: with e = 1 - r2 z and
+    // E = 1 - r2 y0^2, both exact to ~2^-54,
+    //   1 / r = Y = y0 (1 + E / 2 + 3 E^2 / 8),  1 / r^2 = Z = z (1 + e + e^2)
     const V y0 = rsqrt0(P), n0 = neg(y0), z = mul(y0, y0), nze = fma(n0, y0, z), nz = neg(z);  // nze = z - y0^2
-    Tri<V> Y;
+    Tri<V> Y, Z;
     V nf;
     {
         const V nP = neg(P), g = mul(P, z), nge = fma(nP, z, g), f1 = sub(cst(g, 1.f), g);
-        const V pz = mul(P, nze), npe = fma(nP, nze, pz), rz = mul(R2, z), nre = fma(R2, nz, rz);
+        const V rz = mul(R2, z), nre = fma(R3, nz, fma(R2, nz, rz));
         Sum<V> S(cst(g, 0x1p-18f), f1);
         S.put(nge);
-        S.put(pz);
         S.take(rz);
-        V t = sub(add(S.t, nre), npe);
-        t = fma(R2, nze, t);
-        t = fma(R3, nz, t);
-        const V E1 = S.top(), c1 = mul(E1, cst(E1, 0.5f)), q1 = mul(E1, cst(E1, 0.375f)),
-                c2 = fma(q1, E1, mul(t, cst(t, 0.5f)));
-        const V f = mul(y0, c1), nfe = fma(n0, c1, f);
-        Y = {y0, f, sub(mul(y0, c2), nfe)};
+        if constexpr (F) {
+            const V e1 = S.top(), f = mul(z, e1);
+            Z = {z, f, fma(z, fma(e1, e1, add(S.t, nre)), fma(z, e1, neg(f)))};
+        }
+        const V pz = mul(P, nze), npe = fma(nP, nze, pz);  // E = e + r2 (z - y0^2)
+        S.put(pz);
+        const V t = fma(R2, nze, sub(add(S.t, nre), npe));
+        const V E1 = S.top(), yh = mul(y0, cst(y0, 0.5f)), c2 = fma(mul(E1, cst(E1, 0.75f)), E1, t);
+        const V f = mul(yh, E1);
         nf = neg(f);
+        Y = {y0, f, fma(yh, c2, fma(yh, E1, nf))};
     }
     // q / r
     {
@@ -197,26 +196,95 @@ TF_DEV PairTerms<V> pair_terms(const Tri<V> (&x)[3], const Tri<V> (&ny)[3], cons
         o.phi = product(Y, n0, nf, q, p, mul(p, cst(p, 0x1p-18f)));
     }
     if constexpr (!F) return o;
-    // 1 / r^2 = Z
-    Tri<V> Z;
-    {
-        const V m = mul(y0, Y.b), nm = fma(n0, Y.b, m);
-        Sum<V> S(mul(z, cst(z, 0x1p-18f)), mul(m, cst(m, 2.f)));
-        S.take(nze);
-        V t = fma(nm, cst(nm, -2.f), S.t);
-        t = fma(mul(y0, Y.c), cst(t, 2.f), t);
-        t = fma(Y.b, Y.b, t);
-        // z - nze = y0^2
-        Z = {z, S.top(), t};
-    }
-    // W = q / r^3, then W d
     const V w0 = mul(Z.a, o.phi.a);
-    const Tri<V> W = product(Z, nz, neg(Z.b), o.phi, w0, mul(w0, cst(w0, 0x1p-18f)));
-    const V nW = neg(W.a), nWb = neg(W.b), M = mul(W.a, mul(P, mul(y0, cst(y0, 0x1p-18f))));  // 2^-18 |W| r
-#pragma unroll
-    for (int i = 0; i < 3; i++) o.e[i] = product(W, nW, nWb, d[i], mul(W.a, d[i].a), M);
+    o.w = product(Z, nz, neg(Z.b), o.phi, w0, mul(w0, cst(w0, 0x1p-18f)));
     return o;
 }
+
+// The running sums of a target: potential (0) and field (1..3). a takes the
+// terms' leading parts by TwoSums; what is below goes to s, which runs about a
+// constant M far above it and far below the terms (2^-14 of `lim`, itself 1 to 4
+// times the largest term or sum so far), so that three operations add a part
+// and give its rounding error; c takes those. A term's product is not rounded
+// to three floats first: its parts go straight into the sums. Per addition
+// ~2^-58 of the sum is lost (double arithmetic: 2^-54). `settle` after at most
+// 32 terms keeps s near M. (With TwoSums for s as well and the field's products
+// rounded to three floats first, ~365 operations a pair: 200k points 124.5 ms,
+// 110.7 this way.) Sums of 40,000 terms: 2^-53 of the terms' absolute sum at
+// worst, double arithmetic 2^-47.
+template <class V, bool F>
+struct Sums {
+    static constexpr int N = F ? 4 : 1;
+    V a[N], s[N], c[N];
+    float M[2], lim[2];  // of the potential, of the field
+    TF_DEV Sums(V like) {
+#pragma unroll
+        for (int i = 0; i < N; i++) a[i] = s[i] = c[i] = cst(like, 0.f);
+        M[0] = M[1] = lim[0] = lim[1] = 0.f;
+    }
+    TF_DEV V put(int i, V w) {  // s += w; the rounding error
+        const V n = add(s[i], w), r = add(w, sub(s[i], n));
+        s[i] = n;
+        return r;
+    }
+    // terms up to m to come in group g: sums i0 <= i < i1
+    TF_DEV void fit(int g, int i0, int i1, float m) {
+        if (!(m > lim[g])) return;
+        lim[g] = 4.f * m;
+        const float M2 = lim[g] * 0x1p-14f;
+#pragma unroll
+        for (int i = i0; i < i1; i++) {
+            const V b = sub(s[i], cst(s[i], M[g])), n = add(cst(b, M2), b);
+            c[i] = add(c[i], sub(b, sub(n, cst(b, M2))));
+            s[i] = n;
+        }
+        M[g] = M2;
+    }
+    TF_DEV void put_phi(const Tri<V> &x) {
+        fit(0, 0, 1, fmaxf(amax(x.a), amax(a[0])));
+        V e;
+        a[0] = two_sum(a[0], x.a, e);
+        const V r = add(put(0, x.b), put(0, e));
+        c[0] = add(c[0], add(r, x.c));
+    }
+    TF_DEV void put_field(const Tri<V> &W, const Tri<V> (&d)[3]) {
+        const V nW = neg(W.a), nWb = neg(W.b);
+        V p[3];
+        float m = 0.f;
+#pragma unroll
+        for (int i = 0; i < 3; i++) {
+            p[i] = mul(W.a, d[i].a);
+            m = fmaxf(m, fmaxf(amax(p[i]), amax(a[1 + i])));
+        }
+        fit(1, 1, 4, m);
+#pragma unroll
+        for (int i = 0; i < 3; i++) {
+            V e;
+            a[1 + i] = two_sum(a[1 + i], p[i], e);
+            const V m1 = mul(W.a, d[i].b), n1 = fma(nW, d[i].b, m1), m2 = mul(W.b, d[i].a), n2 = fma(nWb, d[i].a, m2);
+            const V pe = fma(W.a, d[i].a, neg(p[i]));
+            V t = add(put(1 + i, m1), put(1 + i, m2));
+            t = add(t, add(put(1 + i, pe), put(1 + i, e)));
+            t = sub(sub(t, n1), n2);
+            t = fma(W.a, d[i].c, t);
+            t = fma(W.b, d[i].b, t);
+            t = fma(W.c, d[i].a, t);
+            c[1 + i] = add(c[1 + i], t);
+        }
+    }
+    TF_DEV void settle() {
+#pragma unroll
+        for (int i = 0; i < N; i++) {
+            const V m = cst(s[i], M[i > 0]);
+            V e;
+            a[i] = two_sum(a[i], sub(s[i], m), e);
+            s[i] = m;
+            const V r = add(c[i], put(i, e)), n = add(s[i], r);
+            c[i] = sub(r, sub(n, s[i]));
+            s[i] = n;
+        }
+    }
+};
 
 }  // namespace tf
 }  // namespace fmm
