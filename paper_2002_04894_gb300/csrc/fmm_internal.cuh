@@ -17,6 +17,7 @@ namespace fmm {
 // or fewer on average, so that a unit's threads are not half idle
 constexpr int kP2PTile = 128;
 constexpr int kP2PTileSmall = 64;
+constexpr int kP2PTileTf = 32;  // FP64 form: a unit is one warp
 // sources per near-field work unit at most (about): a target leaf whose
 // strong list holds more is cut into segments, each its own unit
 constexpr int kP2PSegSources = 1 << 16;
@@ -203,7 +204,7 @@ struct Plan {
     int32_t *p2p_poff = nullptr;
     int64_t p2p_nparts = 0;
     double4 *p2p_partial = nullptr;
-    int p2p_tile = kP2PTile;  // targets per work unit (kP2PTile or kP2PTileSmall)
+    int p2p_tile = kP2PTile;  // targets per work unit (kP2PTile, kP2PTileSmall or kP2PTileTf)
     int32_t *p2p_bstart = nullptr;  // first unit of each of the 256 weight buckets; [256] = units
     bool capacity_exceeded = false;
     // M2L rotation tables (D = d(pi/2) quadrants, axial coefficients, F_nm)

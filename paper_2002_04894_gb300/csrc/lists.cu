@@ -562,8 +562,10 @@ std::atomic<long long> g_list_capacity{0x7fffffffLL};
 // heaviest first). 8 leaves of 125 points: 20.4 us with segments of 256
 // sources, 18.4 with 128.
 static long long p2p_segment(const Plan &P) {
+    // (the FP64 form's single-warp units are counted by the 128 targets of four)
+    const int tile = P.p2p_tile == kP2PTileTf ? kP2PTile : P.p2p_tile;
     const int64_t nl = P.nleaf, want = (int64_t)kP2PUnitsPerSM * sm_count();
-    const int64_t units = nl * std::max<int64_t>(1, (P.n / nl + P.p2p_tile - 1) / P.p2p_tile);
+    const int64_t units = nl * std::max<int64_t>(1, (P.n / nl + tile - 1) / tile);
     if (units >= want) return kP2PSegSources;
     const int64_t k = (want + units - 1) / units;
     const double mean = (double)P.nstrong[P.B] * (double)P.n / ((double)nl * (double)nl);  // sources of a mean list
@@ -672,7 +674,8 @@ cudaError_t lists_build(Plan &P) {
     // added in segment order by the combine pass. The unit and slot totals
     // are read back once to size the arrays.
     const int64_t nl = (int64_t)1 << P.B;
-    P.p2p_tile = (P.prec == FMM_PREC_MIXED && P.n <= (int64_t)kP2PTileSmall * nl) ? kP2PTileSmall : kP2PTile;
+    P.p2p_tile = P.n <= (int64_t)kP2PTileSmall * nl ? kP2PTileSmall : kP2PTile;
+    if (P.prec != FMM_PREC_MIXED) P.p2p_tile = kP2PTileTf;
     const int tile = P.p2p_tile;
     const long long smax = p2p_segment(P);
     P.p2p_work_dev = (unsigned long long *)palloc(P, 24);  // pairs, units, partial slots

@@ -1,15 +1,15 @@
 // Near field of the FP64 form (P2P, Algorithm 4) in three-float arithmetic.
 //
-// What bounds it: the FP32 pipe. A pair takes ~295 packed
-// operations (trifloat.cuh) where FP64 arithmetic takes 19 FP64 instructions at
-// less than two per clock and SM, ~1,400 FP32 operations' time, and its terms
-// are more accurate than those of plain double arithmetic. Sums run in
-// compensated three-float accumulators. 200k Plummer points, 11 levels,
-// 1.16e10 pairs: FP64 arithmetic 412.6 ms (its pipe saturated), this 110.7;
-// 20k uniform points, 8 levels: 3.29 -> 0.95 ms. Registers: 4 blocks of 128
-// threads per SM (128 registers; with ~365 operations a pair 124.5 ms, 5 blocks
-// 127.9, 6 132.7). With block-wide
-// staging and its barriers: 152.9 ms.
+// What bounds it: the FP32 pipe. A pair takes ~295 packed operations
+// (trifloat.cuh) where FP64 arithmetic takes 19 FP64 instructions at less than
+// two per clock and SM, ~1,400 FP32 operations' time, and its terms are more
+// accurate than those of plain double arithmetic. Sums run in compensated
+// three-float accumulators. 200k Plummer points, 11 levels, 1.16e10 pairs: FP64
+// arithmetic 412.6 ms (its pipe saturated), this 107.0; 20k uniform points, 8
+// levels: 3.29 -> 0.96 ms. A unit is one warp and its 32 targets, staging its
+// own sources: units of four warps held their registers until the slowest was
+// done (110.7 ms; with block-wide staging and its barriers slower by a
+// fifth). Registers: 16 warps per SM (128 registers; 18 warps 109.6 ms).
 //
 // Positions are taken relative to the root cell's centre on a common grid of
 // 2^-72 of its extent (rounded up to a power of two): three floats of 24 bits
@@ -141,7 +141,7 @@ k_tf_charges(int64_t n, const double *__restrict__ q, const int *__restrict__ em
     }
 }
 
-constexpr int kT = kP2PTile;  // threads and targets per unit
+constexpr int kT = kP2PTile;  // threads and targets of a block of the direct sum
 constexpr int kChunk = 64;    // sources staged at a time by a warp
 
 // source j on target i in FP64 on the original positions, pairs at zero distance skipped
@@ -159,7 +159,7 @@ __device__ __noinline__ void pair_f64(const double *__restrict__ x, const double
 }
 
 template <typename OutT, bool F>  // F: with the field
-__global__ void __launch_bounds__(kT, 4)
+__global__ void __launch_bounds__(kP2PTileTf, 16)
 k_p2p_tf(int B, int64_t n, const double *__restrict__ x, const double *__restrict__ y, const double *__restrict__ z,
          const double *__restrict__ q, const float *__restrict__ pos, const float *__restrict__ tq,
          const float *__restrict__ thr0, const float *__restrict__ thr, const double *__restrict__ lo,
@@ -168,12 +168,13 @@ k_p2p_tf(int B, int64_t n, const double *__restrict__ x, const double *__restric
          const int32_t *__restrict__ upart, const int32_t *__restrict__ nunits, const int32_t *__restrict__ perm,
          const double *__restrict__ far_phi, const double *__restrict__ far_E, double4 *__restrict__ partial,
          OutT *__restrict__ pot, OutT *__restrict__ field) {
-    // per warp and source pair: parts a, b, c of (x, y, z, q), the two sources
-    // side by side. Each warp stages its own sources: a chunk is some 20,000
-    // cycles of arithmetic, so four warps loading the same one cost nothing,
-    // and none waits for the others at a barrier.
-    __shared__ float4 sm_all[kT / 32][6][kChunk / 2];
-    __shared__ float2 sthr_all[kT / 32][kChunk / 2];
+    // per source pair: parts a, b, c of (x, y, z, q), the two sources side by
+    // side. A unit is one warp: a chunk is some 20,000 cycles of arithmetic, so
+    // several warps loading the same one cost nothing, and the short ones (a
+    // leaf's last targets, sliced over the lanes) give their place up when done.
+    constexpr int kT = kP2PTileTf;
+    __shared__ float4 sm[6][kChunk / 2];
+    __shared__ float2 sthr[kChunk / 2];
     __shared__ double4 red[kT];
     if ((int)blockIdx.x >= *nunits) return;  // launched for an upper bound on the units
     const int64_t off = ((int64_t)1 << B) - 1;
@@ -197,8 +198,6 @@ k_p2p_tf(int B, int64_t n, const double *__restrict__ x, const double *__restric
     if (L.active) thr_i = thr0[slot];
     tf::Sums<float2, F> A(make_float2(0.f, 0.f));
     double slow[4] = {0.0, 0.0, 0.0, 0.0};
-    float4(*sm)[kChunk / 2] = sm_all[tid >> 5];
-    float2 *sthr = sthr_all[tid >> 5];
     float *fs = (float *)sm, *ft = (float *)sthr;
     for (int e = unit.z; e < (busy ? unit.w : 0); e++) {
         const int64_t gs = off + ssrc[e];
@@ -532,7 +531,7 @@ cudaError_t tf_p2p(Plan &P, void *pot, void *field, int dtype) {
     FMM_LAUNCH(k_tf_charges, grid_for(P.n), 256, 0, P.stream, P.n, P.q, P.tf_emax, P.tf_thr0, P.tf_q, P.tf_thr);
     auto go = [&](auto out, auto fld) {  // without a field array only the potential is summed
         using Out = decltype(out);
-        FMM_LAUNCH((k_p2p_tf<Out, decltype(fld)::value>), (unsigned)P.p2p_nunits, kT, 0, P.stream, P.B, P.n, P.x, P.y,
+        FMM_LAUNCH((k_p2p_tf<Out, decltype(fld)::value>), (unsigned)P.p2p_nunits, kP2PTileTf, 0, P.stream, P.B, P.n, P.x, P.y,
                    P.z, P.q, P.tf_pos, P.tf_q, P.tf_thr0, P.tf_thr, P.lo, P.hi, P.tf_emax, P.begin, P.count,
                    P.ssrc[P.B], P.p2p_units, P.p2p_upart, P.p2p_nunits_dev, P.perm, P.far_phi, P.far_E,
                    P.p2p_partial, (Out *)pot, (Out *)field);
