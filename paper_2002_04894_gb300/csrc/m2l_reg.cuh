@@ -291,17 +291,20 @@ __host__ __device__ constexpr int group_first(int n) {  // first degree of degre
 
 // Column sums of degrees G..N over each of the warp's runs of equal target
 // (the pair list is sorted by target; `ends`: the runs' last lanes), added to
-// the run's target's scaled local in double. wt: of several runs, the lanes
-// of the present one as weights 0 or 1, so that a warp with several targets
-// costs a pass per run and not a loop over its lanes.
+// the run's target's scaled local in double. mask: of several runs, the lanes
+// of the present one as bits all 1, the others 0, so that a warp with several
+// targets costs a pass per run and not a loop over its lanes. (Bits and not
+// weights of 0 and 1: another target's sum may hold an infinity.)
 template <int P, int G, int N>
-__device__ __forceinline__ void sum_group(const float *red, float *wt, int t32, unsigned ends,
+__device__ __forceinline__ void sum_group(const float *red, uint32_t *mask, int t32, unsigned ends,
                                           double2 *__restrict__ Lh) {
     constexpr int NC = (P + 1) * (P + 2) / 2, W = (N + 1) * (N + 1) - G * G;
     const int lane = threadIdx.x & 31;
     __syncwarp();
     const bool on = lane < W;
-    const float4 *c4 = (const float4 *)(red + (on ? lane : 0) * kCol), *w4 = (const float4 *)wt;
+    const float4 *c4 = (const float4 *)(red + (on ? lane : 0) * kCol);
+    const uint4 *m4 = (const uint4 *)mask;
+    auto keep = [](float v, uint32_t m) { return __uint_as_float(__float_as_uint(v) & m); };
     int k = G;
 #pragma unroll
     for (int d = G + 1; d <= N; d++) k += lane >= d * d - G * G;
@@ -312,11 +315,11 @@ __device__ __forceinline__ void sum_group(const float *red, float *wt, int t32, 
         const int t = __shfl_sync(0xffffffffu, t32, __ffs(m) - 1);
         if (ends != 0x80000000u) {
             __syncwarp();
-            wt[lane] = t32 == t ? 1.f : 0.f;
+            mask[lane] = t32 == t ? ~0u : 0u;
             __syncwarp();
         }
         float2 a0 = make_float2(0.f, 0.f), a1 = make_float2(0.f, 0.f);
-        if (ends == 0x80000000u) {  // one target: no weights
+        if (ends == 0x80000000u) {  // one target: no mask
 #pragma unroll
             for (int i = 0; i < 8; i++) {
                 const float4 v = c4[i];
@@ -326,9 +329,10 @@ __device__ __forceinline__ void sum_group(const float *red, float *wt, int t32, 
         } else {
 #pragma unroll
             for (int i = 0; i < 8; i++) {
-                const float4 v = c4[i], u = w4[i];
-                a0 = __ffma2_rn(make_float2(v.x, v.y), make_float2(u.x, u.y), a0);
-                a1 = __ffma2_rn(make_float2(v.z, v.w), make_float2(u.z, u.w), a1);
+                const float4 v = c4[i];
+                const uint4 u = m4[i];
+                a0 = __fadd2_rn(a0, make_float2(keep(v.x, u.x), keep(v.y, u.y)));
+                a1 = __fadd2_rn(a1, make_float2(keep(v.z, u.z), keep(v.w, u.w)));
             }
         }
         const float s = (a0.x + a0.y) + (a1.x + a1.y);
@@ -339,8 +343,8 @@ __device__ __forceinline__ void sum_group(const float *red, float *wt, int t32, 
 
 // inverse rotation of degree N into the transpose buffer, scaled by tp = qt^N / rho
 template <int P, int N>
-__device__ __forceinline__ void inv(State<P> &S, const float2 *za, const float2 *zb, float tp, float *red, float *wt,
-                                    int t32, unsigned ends, double2 *__restrict__ Lh) {
+__device__ __forceinline__ void inv(State<P> &S, const float2 *za, const float2 *zb, float tp, float *red,
+                                    uint32_t *mask, int t32, unsigned ends, double2 *__restrict__ Lh) {
     constexpr int c0 = N * (N + 1) / 2, G = group_first(N);
     if constexpr (N >= sync_from<P>()) __syncthreads();
     float ur[N + 1], ui[N + 1], xr[N + 1], xi[N + 1];
@@ -356,10 +360,10 @@ __device__ __forceinline__ void inv(State<P> &S, const float2 *za, const float2 
         col[l * kCol] = ur[l];
         if (l) col[(N + l) * kCol] = ui[l];
     }
-    if constexpr (N == P || group_first(N + 1) != G) sum_group<P, G, N>(red, wt, t32, ends, Lh);
+    if constexpr (N == P || group_first(N + 1) != G) sum_group<P, G, N>(red, mask, t32, ends, Lh);
 }
 
-// bytes of a warp's slice of shared memory: its source rows, the run's weights, the transpose buffer, the mbarrier of the copies
+// bytes of a warp's slice of shared memory: its source rows, the run's mask, the transpose buffer, the mbarrier of the copies
 template <int P>
 __host__ __device__ constexpr int slice_bytes() {
     return 32 * row_bytes(P) + 128 + 4 * kCol * ((P + 1) * (P + 1) < 32 ? (P + 1) * (P + 1) : 32) + 16;
@@ -377,7 +381,7 @@ constexpr size_t smem_bytes() { return (size_t)slice_bytes<P>() * warps<P>(); }
 struct Cursor {
     int gt, gs;   // target and source box of this lane's pair
     int sys;      // system (batched)
-    bool valid;   // lanes past the end repeat the last pair with weight zero
+    bool valid;   // lanes past the end repeat the last pair, for no target
 };
 
 // the pairs of one plan
@@ -444,7 +448,8 @@ __device__ __forceinline__ void run(Src &src, char *slice) {
     unsigned w0 = blockIdx.x * W;  // the block's first chunk (device memory holds fewer than 2^31 chunks of pairs)
     if (w0 >= total) return;
     const char *rowp = slice + (threadIdx.x & 31) * row_bytes(P);
-    float *wt = (float *)(slice + 32 * row_bytes(P)), *red = wt + 32;
+    uint32_t *mask = (uint32_t *)(slice + 32 * row_bytes(P));
+    float *red = (float *)(mask + 32);
     Cursor nxt = src.at(w0 + (threadIdx.x >> 5));
     float4 th, tl, sh, sl;  // split centres and radii of the next target and source box
     auto geometry = [&](const Cursor &c) {
@@ -512,16 +517,16 @@ __device__ __forceinline__ void run(Src &src, char *slice) {
             Phases<P> A, B;
             A.set(eai);
             B.set(eb);
-            float tp = cur.valid ? rinv : 0.f;
-            const int up = __shfl_down_sync(0xffffffffu, cur.gt, 1);
-            const unsigned ends = __ballot_sync(0xffffffffu, (threadIdx.x & 31) == 31 || up != cur.gt);
+            float tp = rinv;
+            const int t32 = cur.valid ? cur.gt : -1, up = __shfl_down_sync(0xffffffffu, t32, 1);
+            const unsigned ends = __ballot_sync(0xffffffffu, cur.valid && ((threadIdx.x & 31) == 31 || up != t32));
             double2 *Lh = src.Lh(cur);
             static_for<P + 1>([&](auto n) {
                 constexpr int N = decltype(n)::value;
                 if constexpr (N == (P * 9 + 9) / 10) {
                     if (more) geometry(nxt);
                 }
-                inv<P, N>(S, A.z, B.z, tp, red, wt, cur.gt, ends, Lh);
+                inv<P, N>(S, A.z, B.z, tp, red, mask, t32, ends, Lh);
                 tp *= qt;
             });
         }

@@ -60,3 +60,28 @@ def test_batch_equals_alone(gpu_lib, p):
         fmm.fmm_eval_check(plan)
         # the same sums in another order of the double atomics: a float ulp or two (as the other batch tests hold)
         assert float((a - b).norm() / a.norm()) <= 1e-6
+
+
+@pytest.mark.parametrize("p", [2, 4])
+def test_overflow_stays_with_its_target(gpu_lib, p):
+    """A charge so large that its M2L into the boxes near it overflows in single
+    precision, in a long thin box whose far end it reaches with finite values: the
+    targets there, which share warps with the overflowing ones, are not touched.
+    Tolerance against the FP64 form: as above for the expansions, and as much again
+    for the near field's runs and L2P."""
+    fmm = gpu_lib
+    n = 3000
+    xn = inputs.points("uniform", n, seed=p) * np.array([0.03, 3e-4, 3e-4])
+    xn[0] = [0.0, 1.5e-4, 1.5e-4]
+    qn = inputs.charges_uniform(n, seed=p) * 1e30
+    qn[0] = 1e36
+    x, q = torch.from_numpy(xn).cuda(), torch.from_numpy(qn).cuda()
+    pot = []
+    for prec in (fmm.FMM_PREC_FP64, fmm.FMM_PREC_MIXED):
+        plan = fmm.fmm_plan(x, 9, p, 0.5, prec=prec)
+        pot.append(fmm.fmm_eval(plan, q)[0].cpu().numpy())
+    far = xn[:, 0] > 0.0125                    # potentials of 3.3e37 to 8e37
+    assert far.sum() > 1000
+    assert not np.isfinite(fmm.fmm_eval_expansions(plan, "L")).all()   # (the overflow does happen)
+    err = np.abs(pot[1][far] - pot[0][far]).max() / np.abs(pot[0][far]).max()
+    assert err <= 2 * (5 * (p + 1) + 16) * 2.0 ** -24, err
