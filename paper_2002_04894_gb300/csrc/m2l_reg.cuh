@@ -255,7 +255,11 @@ __device__ __forceinline__ void fwd(const char *rowp, const float2 *za, const fl
     }
 }
 
-// translation along z of order L, in place
+// Translation along z of order L, in place. The terms fall with the degree (by
+// (r_s / rho)^n), so the sums run from the highest degree down: a chain that
+// starts from the small terms loses half as much as one that starts from the
+// large ones (potential of a pair's translation, p = 12: 3.7e-8 against 7.2e-8
+// relative; two chains added at the end 6.1e-8).
 template <int P, int L>
 __device__ __forceinline__ void axial(State<P> &S) {
     float sr[P + 1 - L], si[P + 1 - L];
@@ -265,10 +269,10 @@ __device__ __forceinline__ void axial(State<P> &S) {
         constexpr int K = L + decltype(kk)::value, c = K * (K + 1) / 2 + L;
         float a = 0.f, b = 0.f;
         static_for<P + 1 - L>([&](auto nn) {
-            constexpr int j = decltype(nn)::value;
+            constexpr int j = P - L - decltype(nn)::value;
             constexpr float w = Axial<L, K, L + j>::v;
-            a = j == 0 ? w * sr[j] : fmaf(w, sr[j], a);
-            if constexpr (L > 0) b = j == 0 ? w * si[j] : fmaf(w, si[j], b);
+            a = j == P - L ? w * sr[j] : fmaf(w, sr[j], a);
+            if constexpr (L > 0) b = j == P - L ? w * si[j] : fmaf(w, si[j], b);
         });
         S.r[c] = a;
         if constexpr (L > 0) S.i[c] = b;

@@ -85,3 +85,35 @@ def test_overflow_stays_with_its_target(gpu_lib, p):
     assert not np.isfinite(fmm.fmm_eval_expansions(plan, "L")).all()   # (the overflow does happen)
     err = np.abs(pot[1][far] - pot[0][far]).max() / np.abs(pot[0][far]).max()
     assert err <= 2 * (5 * (p + 1) + 16) * 2.0 ** -24, err
+
+
+@pytest.mark.parametrize("p", [8, 12])
+def test_constant_term_of_one_pair(gpu_lib, p):
+    """What the axial sum loses in a local expansion's constant term: two clusters of
+    positive charges, one weak pair each way. Half the difference of the two boxes'
+    relative errors, each less its source's monopole's, is free of the roundings both
+    share (the distance's reciprocal) and of P2M's. The sum's terms fall with the
+    degree, and one chain from the smallest up is to lose less than two chains added
+    at the end (as orders 14 and 16 sum). Tolerance, from an emulation of the same
+    20,000 pairs' roundings (root mean square in 2^-24): 0.73 with two chains, 0.91
+    with one from the largest down, 0.44 from the smallest up."""
+    fmm = gpu_lib
+    rng = np.random.default_rng(p)
+    half = []
+    for _ in range(200):
+        d = rng.normal(size=3)
+        d *= 2.0 / rng.uniform(0.3, 0.45) / np.linalg.norm(d)
+        xn = rng.uniform(-1, 1, (80, 3)) / np.sqrt(3.0)
+        xn[40:] += d
+        x, q = torch.from_numpy(xn).cuda(), torch.from_numpy(rng.uniform(0, 1, 80)).cuda()
+        got = {}
+        for prec in (fmm.FMM_PREC_FP64, fmm.FMM_PREC_MIXED):
+            plan = fmm.fmm_plan(x, 1, p, 0.5, prec=prec, tight=True)
+            fmm.fmm_eval(plan, q)
+            assert fmm.fmm_plan_stats(plan)["weak_pairs"] == 2
+            got[prec] = [fmm.fmm_eval_expansions(plan, w)[1:, 0].real for w in "LM"]
+        (l0, m0), (l1, m1) = got[fmm.FMM_PREC_FP64], got[fmm.FMM_PREC_MIXED]
+        e = (l1 / l0 - 1) - (m1 / m0 - 1)[::-1]
+        half.append((e[0] - e[1]) / 2)
+    rms = np.sqrt(np.mean(np.square(half)))
+    assert rms <= 0.73 * 2.0 ** -24, rms * 2.0 ** 24
