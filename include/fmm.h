@@ -202,11 +202,13 @@ void fmm_destroy(fmm_plan_t plan);
  *   points, charges  n x 3 and n values (dtype), host or device.
  *   targets          ntargets int64 indices into [0, n), host or device.
  *   potentials       ntargets outputs (dtype); fields: ntargets x 3 or NULL.
- * The pairs run in three-float arithmetic with compensated sums (relative
- * errors below those of double arithmetic), pairs it cannot hold in double.
- * Takes its workspace (up to about 58 MB, and 32 bytes per target and source
- * segment) from the library's stream-ordered pool and gives it back before it
- * returns; device staging for host arguments with cudaMallocAsync.
+ * The pairs run in three-float arithmetic (terms and sums of 1,000 more exact
+ * than double arithmetic's), pairs it cannot hold in double; all further sums
+ * are compensated (Neumaier).
+ * Takes its workspace (up to about 58 MB, and 64 bytes per target and source
+ * segment) from the library's stream-ordered pool. It goes back to that pool,
+ * which keeps the memory for later calls until fmm_pool_trim. Device staging
+ * for host arguments with cudaMallocAsync.
  * Errors: FMM_EINVAL (n < 1, ntargets < 0, NULL pointers), FMM_ECUDA.
  */
 int fmm_direct(const void *points, const void *charges, int64_t n, int dtype,

@@ -115,9 +115,10 @@ struct P2PLane {
             }
         }
     }
-    // The slices' sums added in slice order (block-wide call; `buf` holds one
-    // double4 per thread). Returns whether this thread owns a target's sum.
-    __device__ __forceinline__ bool combine(double4 &v, double4 *buf) const {
+    // The slices' sums added in slice order, v = add(v, other) (block-wide call;
+    // `buf` holds one V per thread). Returns whether this thread owns a target's sum.
+    template <class V, class Add>
+    __device__ __forceinline__ bool combine(V &v, V *buf, Add &&add) const {
         if (rest <= left) return active;  // one slice each (uniform over the block)
         const int k = (int)threadIdx.x - first;
         __syncthreads();
@@ -125,16 +126,28 @@ struct P2PLane {
         __syncthreads();
         if (k < 0) return active;
         if (k >= left) return false;
-        for (int j = k + left; j < rest; j += left) {
-            const double4 o = buf[j];
-            v.x += o.x;
-            v.y += o.y;
-            v.z += o.z;
-            v.w += o.w;
-        }
+        for (int j = k + left; j < rest; j += left) add(v, buf[j]);
         return true;
     }
+    __device__ __forceinline__ bool combine(double4 &v, double4 *buf) const {
+        return combine(v, buf, [](double4 &a, const double4 &o) {
+            a.x += o.x;
+            a.y += o.y;
+            a.z += o.z;
+            a.w += o.w;
+        });
+    }
 };
+
+// s + c += v, the rounding error of s into c (Neumaier)
+__device__ __forceinline__ void neumaier(double &s, double &c, double v) {
+    const double t = s + v;
+    if (fabs(s) >= fabs(v))
+        c += (s - t) + v;
+    else
+        c += (v - t) + s;
+    s = t;
+}
 
 // Block b of a batched launch belongs to system s with off[s] <= b < off[s+1].
 __device__ __forceinline__ int batch_sys_of(const int32_t *__restrict__ off, int nsys, int64_t b) {

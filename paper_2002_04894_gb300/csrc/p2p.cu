@@ -17,15 +17,6 @@ namespace fmm {
 
 namespace {
 
-__device__ __forceinline__ void neumaier(double &s, double &c, double v) {
-    const double t = s + v;
-    if (fabs(s) >= fabs(v))
-        c += (s - t) + v;
-    else
-        c += (v - t) + s;
-    s = t;
-}
-
 template <typename T>
 __global__ void __launch_bounds__(256)
 k_direct(const T *__restrict__ pts, const T *__restrict__ q, int64_t n,

@@ -279,12 +279,18 @@ k_p2p_tf(int B, int64_t n, const double *__restrict__ x, const double *__restric
 // y, z, q, then the thresholds; every lane of a warp reads the same record), a
 // slab of them at a time; a block takes 128 targets against a segment of the
 // slab and adds its sums to the (segment, target) slot; a last pass adds the
-// segments. 500k points, 1000 targets (5e8 pairs): one block per target in FP64
+// segments. Everything outside the three floats' own sums (pairs left to FP64,
+// those sums every kFlush records, slices, slabs, segments) is added in doubles
+// with Neumaier's compensation: with one segment a target's sum runs over the
+// whole slab (100,000 targets, all pairs left to FP64: ~4e-15 relative without
+// it). 500k points, 1000 targets (5e8 pairs): one block per target in FP64
 // arithmetic (square root, two divisions and Neumaier sums a pair) 58.6 ms,
-// this 4.92 (~295 operations a pair; ~365: 5.48); 1 target:
-// 8.40 -> 0.36 ms, 2000 points and 1000 targets 0.38 -> 0.08.
+// this 5.00 (4.92 with plain sums; ~365 instead of ~295 operations a pair: 5.48);
+// all pairs left to FP64 51.8; 1 target: 8.40 -> 0.36 ms, 2000 points and 1000
+// targets 0.38 -> 0.08.
 // ---------------------------------------------------------------------------
 constexpr int kRec = 7;
+constexpr int kFlush = 1024;  // records between flushes: three-float sums of 1000 terms hold 2^-57 of them, of 10^6 2^-51
 constexpr int64_t kSlab = 1 << 20;  // sources split at a time (58 MB of records)
 
 // the grid of the points: centre, 2^-k, whether it holds (grid_exponent), and the charges' exponent
@@ -397,19 +403,45 @@ k_direct_split(const T *__restrict__ pts, const T *__restrict__ q, int64_t n, in
     }
 }
 
+// compensated sums of the potential and the field
+struct Sum4 {
+    double s[4], c[4];
+    __device__ __forceinline__ void add(const Sum4 &o) {
+#pragma unroll
+        for (int i = 0; i < 4; i++) {
+            neumaier(s[i], c[i], o.s[i]);
+            c[i] += o.c[i];
+        }
+    }
+    // (an infinite sum has no correction)
+    __device__ __forceinline__ double get(int i) const { return isfinite(s[i]) ? s[i] + c[i] : s[i]; }
+};
+
 // source j on target i in FP64, pairs at zero distance skipped
 template <typename T>
 __device__ __noinline__ void direct_f64(const T *__restrict__ pts, const T *__restrict__ q, int64_t i, int64_t j,
-                                        double (&s)[4]) {
+                                        Sum4 &s) {
     const double dx = (double)pts[3 * i] - (double)pts[3 * j], dy = (double)pts[3 * i + 1] - (double)pts[3 * j + 1],
                  dz = (double)pts[3 * i + 2] - (double)pts[3 * j + 2];
     const double r2 = dx * dx + dy * dy + dz * dz;
     if (r2 == 0.0) return;
     const double r = sqrt(r2), qj = (double)q[j], qr3 = qj / (r2 * r);
-    s[0] += qj / r;
-    s[1] += qr3 * dx;
-    s[2] += qr3 * dy;
-    s[3] += qr3 * dz;
+    neumaier(s.s[0], s.c[0], qj / r);
+    neumaier(s.s[1], s.c[1], qr3 * dx);
+    neumaier(s.s[2], s.c[2], qr3 * dy);
+    neumaier(s.s[3], s.c[3], qr3 * dz);
+}
+
+// A, sums of positions over 2^k and charges over 2^eq, added to S
+__device__ __forceinline__ void flush(const tf::Sums<float2, true> &A, int k, int eq, Sum4 &S) {
+#pragma unroll
+    for (int i = 0; i < 4; i++) {
+        const int e = i ? eq - 2 * k : eq - k;
+        const double m = A.M[i > 0];
+        neumaier(S.s[i], S.c[i], scalbn(((double)A.a[i].x + (double)A.a[i].y) +
+                                            ((((double)A.s[i].x - m) + ((double)A.s[i].y - m)) +
+                                             ((double)A.c[i].x + (double)A.c[i].y)), e));
+    }
 }
 
 // block (x: targets 128 x .., y: records [y len, (y + 1) len) of the slab)
@@ -417,8 +449,8 @@ template <typename T>
 __global__ void __launch_bounds__(kT, 4)
 k_direct_tf(const T *__restrict__ pts, const T *__restrict__ q, int64_t n, const int64_t *__restrict__ targets,
             int64_t nt, int64_t j0, int64_t j1, const DirectBox *__restrict__ box, const float4 *__restrict__ rec,
-            int64_t len, bool first, double4 *__restrict__ partial) {
-    __shared__ double4 red[kT];
+            int64_t len, bool first, Sum4 *__restrict__ partial) {
+    __shared__ Sum4 red[kT];
     const int64_t t0 = (int64_t)blockIdx.x * kT;
     const P2PLane L((int)min((int64_t)kT, nt - t0), kT, threadIdx.x);
     const int64_t i = L.active ? targets[t0 + L.target] : -1;
@@ -430,82 +462,76 @@ k_direct_tf(const T *__restrict__ pts, const T *__restrict__ q, int64_t n, const
 #pragma unroll
     for (int a = 0; a < 3; a++)
         X[a] = {make_float2(f[a][0], f[a][0]), make_float2(f[a][1], f[a][1]), make_float2(f[a][2], f[a][2])};
-    tf::Sums<float2, true> A(make_float2(0.f, 0.f));
-    double slow[4] = {0.0, 0.0, 0.0, 0.0};
+    Sum4 S = {};
     const int64_t np = (j1 - j0 + 1) >> 1, p1 = busy ? min(np, (blockIdx.y + 1) * len) : 0;
 #pragma unroll 1
-    for (int64_t pp = blockIdx.y * len + L.slice, terms = 1; pp < p1; pp += L.slices, terms++) {
-        const float4 *r = rec + pp * kRec;
-        const float4 a0 = __ldg(r), a1 = __ldg(r + 1), b0 = __ldg(r + 2), b1 = __ldg(r + 3), c0 = __ldg(r + 4),
-                     c1 = __ldg(r + 5), th = __ldg(r + 6);
-        const tf::Tri<float2> Y[3] = {{make_float2(a0.x, a0.y), make_float2(b0.x, b0.y), make_float2(c0.x, c0.y)},
-                                      {make_float2(a0.z, a0.w), make_float2(b0.z, b0.w), make_float2(c0.z, c0.w)},
-                                      {make_float2(a1.x, a1.y), make_float2(b1.x, b1.y), make_float2(c1.x, c1.y)}};
-        const tf::Tri<float2> Q = {make_float2(a1.z, a1.w), make_float2(b1.z, b1.w), make_float2(c1.z, c1.w)};
-        tf::PairTerms<float2> o = tf::pair_terms(X, Y, Q);
-        const bool bx = o.r2.x < fmaxf(th.x, thr_i), by = o.r2.y < fmaxf(th.y, thr_i);
-        if (bx || by) {
-            const int64_t j = j0 + 2 * pp;
-            if (bx) {
-                if (on && (j != i || isinf(th.x))) direct_f64(pts, q, i, j, slow);
-                clear_x(o);
+    for (int64_t pp = blockIdx.y * len + L.slice; pp < p1;) {
+        tf::Sums<float2, true> A(make_float2(0.f, 0.f));
+        const int64_t end = min(p1, pp + kFlush * L.slices);
+#pragma unroll 1
+        for (int terms = 1; pp < end; pp += L.slices, terms++) {
+            const float4 *r = rec + pp * kRec;
+            const float4 a0 = __ldg(r), a1 = __ldg(r + 1), b0 = __ldg(r + 2), b1 = __ldg(r + 3), c0 = __ldg(r + 4),
+                         c1 = __ldg(r + 5), th = __ldg(r + 6);
+            const tf::Tri<float2> Y[3] = {{make_float2(a0.x, a0.y), make_float2(b0.x, b0.y), make_float2(c0.x, c0.y)},
+                                          {make_float2(a0.z, a0.w), make_float2(b0.z, b0.w), make_float2(c0.z, c0.w)},
+                                          {make_float2(a1.x, a1.y), make_float2(b1.x, b1.y), make_float2(c1.x, c1.y)}};
+            const tf::Tri<float2> Q = {make_float2(a1.z, a1.w), make_float2(b1.z, b1.w), make_float2(c1.z, c1.w)};
+            tf::PairTerms<float2> o = tf::pair_terms(X, Y, Q);
+            const bool bx = o.r2.x < fmaxf(th.x, thr_i), by = o.r2.y < fmaxf(th.y, thr_i);
+            if (bx || by) {
+                const int64_t j = j0 + 2 * pp;
+                if (bx) {
+                    if (on && (j != i || isinf(th.x))) direct_f64(pts, q, i, j, S);
+                    clear_x(o);
+                }
+                if (by) {
+                    if (on && j + 1 < j1 && (j + 1 != i || isinf(th.y))) direct_f64(pts, q, i, j + 1, S);
+                    clear_y(o);
+                }
             }
-            if (by) {
-                if (on && j + 1 < j1 && (j + 1 != i || isinf(th.y))) direct_f64(pts, q, i, j + 1, slow);
-                clear_y(o);
-            }
+            A.put_phi(o.phi);
+            A.put_field(o.w, o.d);
+            if ((terms & 31) == 0) A.settle();
         }
-        A.put_phi(o.phi);
-        A.put_field(o.w, o.d);
-        if ((terms & 31) == 0) A.settle();
+        A.settle();
+        flush(A, box->grid.k, box->grid.eq, S);
     }
-    A.settle();
-    double4 r = result(A, slow, box->grid.k, box->grid.eq);
-    if (L.combine(r, red)) {
-        double4 *slot = partial + blockIdx.y * nt + t0 + L.target;
-        if (!first) {
-            const double4 o = *slot;
-            r.x += o.x;
-            r.y += o.y;
-            r.z += o.z;
-            r.w += o.w;
-        }
-        *slot = r;
+    if (L.combine(S, red, [](Sum4 &a, const Sum4 &o) { a.add(o); })) {
+        Sum4 *slot = partial + blockIdx.y * nt + t0 + L.target;
+        if (!first) S.add(*slot);
+        *slot = S;
     }
 }
 
 template <typename T>
 __global__ void __launch_bounds__(256)
 k_direct_finish(int64_t n, const int64_t *__restrict__ targets, int64_t nt, int64_t segs,
-                const double4 *__restrict__ partial, T *__restrict__ pot, T *__restrict__ field) {
+                const Sum4 *__restrict__ partial, T *__restrict__ pot, T *__restrict__ field) {
     // a warp per target, the lanes over the segments
     const int lane = threadIdx.x & 31;
     for (int64_t t = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; t < nt;
          t += ((int64_t)gridDim.x * blockDim.x) >> 5) {
-        double4 r = make_double4(0.0, 0.0, 0.0, 0.0);
-        for (int64_t s = lane; s < segs; s += 32) {
-            const double4 o = partial[s * nt + t];
-            r.x += o.x;
-            r.y += o.y;
-            r.z += o.z;
-            r.w += o.w;
-        }
+        Sum4 r = {};
+        for (int64_t s = lane; s < segs; s += 32) r.add(partial[s * nt + t]);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
-            r.x += __shfl_xor_sync(0xffffffffu, r.x, o);
-            r.y += __shfl_xor_sync(0xffffffffu, r.y, o);
-            r.z += __shfl_xor_sync(0xffffffffu, r.z, o);
-            r.w += __shfl_xor_sync(0xffffffffu, r.w, o);
+            Sum4 v;
+#pragma unroll
+            for (int i = 0; i < 4; i++) {
+                v.s[i] = __shfl_xor_sync(0xffffffffu, r.s[i], o);
+                v.c[i] = __shfl_xor_sync(0xffffffffu, r.c[i], o);
+            }
+            r.add(v);
         }
         if (lane) continue;
         const int64_t i = targets[t];
-        if (i < 0 || i >= n) r.x = r.y = r.z = r.w = __longlong_as_double(0x7ff8000000000000ll);
-        pot[t] = (T)r.x;
-        if (field) {
-            field[3 * t] = (T)r.y;
-            field[3 * t + 1] = (T)r.z;
-            field[3 * t + 2] = (T)r.w;
-        }
+        const bool ok = i >= 0 && i < n;
+        const double nan = __longlong_as_double(0x7ff8000000000000ll);
+        pot[t] = (T)(ok ? r.get(0) : nan);
+        if (field)
+#pragma unroll
+            for (int a = 0; a < 3; a++) field[3 * t + a] = (T)(ok ? r.get(1 + a) : nan);
     }
 }
 
@@ -551,12 +577,12 @@ static cudaError_t direct_tf_run(const T *pts, const T *q, int64_t n, const int6
     const int64_t want = std::max<int64_t>(1, 16 * (int64_t)sm_count() / tiles);
     const int64_t len = std::max<int64_t>(64, (recs + want - 1) / want);
     const int64_t segs = std::min<int64_t>((recs + len - 1) / len, 65535), len1 = (recs + segs - 1) / segs;
-    const size_t b0 = 512, b1 = (size_t)recs * kRec * 16, b2 = (size_t)segs * nt * sizeof(double4);
+    const size_t b0 = 512, b1 = (size_t)recs * kRec * 16, b2 = (size_t)segs * nt * sizeof(Sum4);
     char *w = (char *)pool_alloc(b0 + ((b1 + 255) & ~(size_t)255) + b2, st);
     if (!w) return cudaErrorMemoryAllocation;
     DirectBox *box = (DirectBox *)w;
     float4 *rec = (float4 *)(w + b0);
-    double4 *partial = (double4 *)(w + b0 + ((b1 + 255) & ~(size_t)255));
+    Sum4 *partial = (Sum4 *)(w + b0 + ((b1 + 255) & ~(size_t)255));
     FMM_LAUNCH(k_direct_box_init, 1, 32, 0, st, box);
     FMM_LAUNCH(k_direct_box<T>, grid_for(n), 256, 0, st, pts, q, n, box);
     for (int64_t j0 = 0; j0 < n; j0 += kSlab) {

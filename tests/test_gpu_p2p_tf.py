@@ -101,3 +101,24 @@ def test_direct_slabs_and_bad_indices(gpu_lib):
         assert abs(pot[k] - (w * Q).sum()) <= 2.0 ** -23 * abs((w * Q).sum()) + 1e-12 * (w * abs(Q)).sum()
         E = ((w ** 3 * Q)[:, None] * d).sum(0)
         assert np.all(abs(fld[k] - E) <= 2.0 ** -23 * abs(E) + 1e-12 * (w ** 2 * abs(Q)).sum())
+
+
+def test_direct_long_sums_of_pairs_left_to_fp64(gpu_lib):
+    """A far outlier (every pair of the cluster is then left to FP64) and many targets
+    (few segments: a thread adds some 30,000 terms of one sign). Tolerance: the terms'
+    own roundings in FP64, at most 4 2^-53 of 1/r and 11 2^-53 of d/r^3, and 2 2^-53
+    for compensated sums and the result."""
+    fmm = gpu_lib
+    n = 100_000
+    rng = np.random.default_rng(29)
+    x, q = rng.random((n, 3)), rng.uniform(0.5, 1.0, n)
+    x[0] = 1e8, 0.0, 0.0
+    pot, fld = (v.cpu().numpy() for v in fmm.fmm_direct(torch.from_numpy(x).cuda(), torch.from_numpy(q).cuda(),
+                                                        torch.arange(n, device="cuda")))
+    X, Q = x.astype(np.longdouble), q.astype(np.longdouble)
+    for t in range(1, n, n // 12):
+        d = X[t] - X
+        r = np.sqrt((d * d).sum(1))
+        w = np.divide(np.longdouble(1), r, out=np.zeros_like(r), where=r > 0)
+        assert abs(pot[t] - (w * Q).sum()) <= 6 * 2.0 ** -53 * (w * Q).sum()
+        assert np.all(abs(fld[t] - ((w ** 3 * Q)[:, None] * d).sum(0)) <= 13 * 2.0 ** -53 * (w ** 2 * Q).sum())
