@@ -93,11 +93,13 @@ def batch_copies(n: int, points: int = 1_000_000, cap: int = 128) -> int:
 
 
 def tune(points, charges, tol: float = 1e-6, leaf_range=(32, 256), thetas=(0.4, 0.5, 0.6),
-         ps=(6, 8, 10, 12, 14, 16), prec=None, targets: int = 300, seed: int = 0, batch: int = 0) -> TuneResult:
+         ps=(6, 8, 10, 12, 14, 16), prec=None, targets: int = 300, seed: int = 0, batch: int = 0, fields: bool = True) -> TuneResult:
     """Search (levels, theta, p) for the fastest solve meeting `tol` (relative
     L2 potential error against the FP64 direct sum on sampled targets).
     batch > 0: the cost is the evaluation time per system in a batch of
-    `batch` copies (one launch per stage)."""
+    `batch` copies (one launch per stage). fields: whether the evaluations to
+    come ask for the field (without it a near-field pair costs about half, and
+    larger leaves pay)."""
     import numpy as np
     import torch
 
@@ -117,7 +119,8 @@ def tune(points, charges, tol: float = 1e-6, leaf_range=(32, 256), thetas=(0.4, 
         from .serve import build_plans
         plans = build_plans([xd] * batch, [cfg] * batch, prec=prec)
         pots = [torch.empty(n, dtype=qd.dtype, device=qd.device) for _ in range(batch)]
-        b = fmm_batch_create(plans, [qd] * batch, pots)
+        flds = [torch.empty((n, 3), dtype=qd.dtype, device=qd.device) for _ in range(batch)] if fields else None
+        b = fmm_batch_create(plans, [qd] * batch, pots, flds)
         times = []
         for _ in range(3):
             e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
@@ -142,7 +145,7 @@ def tune(points, charges, tol: float = 1e-6, leaf_range=(32, 256), thetas=(0.4, 
             a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
             a.record()
             plan = fmm_plan(xd, cfg.levels, cfg.p, cfg.theta, prec=prec)
-            pot, _ = fmm_eval(plan, qd, want_fields=False)
+            pot, _ = fmm_eval(plan, qd, want_fields=fields)
             b.record()
             torch.cuda.synchronize()
             times.append(a.elapsed_time(b))

@@ -210,6 +210,31 @@ def test_tuner_meets_target(gpu_lib, batch):
     assert r.config.theta in (0.4, 0.5, 0.6)
 
 
+@pytest.mark.parametrize("fields", [None, True, False])
+@pytest.mark.parametrize("batch", [0, 4])
+def test_tuner_times_the_evaluation_that_will_run(gpu_lib, monkeypatch, batch, fields):
+    """Every trial asks for the field exactly when the evaluations to come do (by default they do)."""
+    fmm, asked = gpu_lib, []
+    plain_eval, plain_create = fmm.fmm_eval, fmm.fmm_batch_create
+
+    def spy_eval(plan, q, want_fields=True, **kw):
+        asked.append(want_fields)
+        return plain_eval(plan, q, want_fields=want_fields, **kw)
+
+    def spy_create(plans, charges, potentials, flds=None, **kw):
+        asked.append(flds is not None and all(f.shape == (4000, 3) for f in flds))
+        return plain_create(plans, charges, potentials, flds, **kw)
+
+    monkeypatch.setattr(fmm, "fmm_eval", spy_eval)
+    monkeypatch.setattr(fmm, "fmm_batch_create", spy_create)
+    x = torch.from_numpy(inputs.points("plummer", 4000, 3)).cuda()
+    q = torch.from_numpy(inputs.charges_uniform(4000, 3)).cuda()
+    kw = {} if fields is None else {"fields": fields}
+    r = tune.tune(x, q, tol=1e-4, ps=(6, 8), batch=batch, **kw)
+    assert len(asked) >= len(r.trials) > 0
+    assert set(asked) == {fields is not False}
+
+
 def test_server_resident_plans_equal_fresh_solves(gpu_lib):
     """Requests naming their point set (geom) reuse a resident plan with new
     charges: each result equals a fresh solve of the same points and charges,
