@@ -325,11 +325,18 @@ k_lists_head(int last, int step, double theta, const double *__restrict__ centre
     }
 }
 
+// segments of a strong list of len entries holding ns sources: one per smax of
+// them, no more than there are entries to cut between
+__device__ __forceinline__ int p2p_segments(unsigned long long ns, long long smax, int len) {
+    const unsigned long long k = (ns + (unsigned long long)smax - 1) / (unsigned long long)smax;
+    return (int)max(1ull, min(k, (unsigned long long)len));
+}
+
 // per target leaf the near source points (sum of n_s over its strong leaf
 // pairs), and in total the sum over strong leaf pairs (t, s) of n_t * n_s.
 // Per leaf: its sources over the strong list, its number of near-field work
-// units -- tiles of `tile` targets times k source segments, k = ceil(sources /
-// smax) -- and, when k > 1, the k * n_t partial-sum slots its split units fill;
+// units -- tiles of `tile` targets times k source segments (p2p_segments) --
+// and, when k > 1, the k * n_t partial-sum slots its split units fill;
 // the totals (pairs, units, slots) into acc[0..2] in 64 bits. One warp per
 // leaf, its lanes striding over the strong list (lists of large boxes in
 // sparse regions hold a good part of the tree).
@@ -351,7 +358,7 @@ __global__ void k_p2p_work(int B, int tile, long long smax, const int32_t *sptr,
         if (lane == 0) {
             const int n_t = count[off + t];
             per_leaf[t] = (long long)ns;
-            const unsigned long long k = ns > (unsigned long long)smax ? (ns + smax - 1) / smax : 1;
+            const unsigned long long k = (unsigned long long)p2p_segments(ns, smax, e1 - sptr[t]);
             const unsigned long long u = (unsigned long long)((n_t + tile - 1) / tile) * k;
             const unsigned long long pp = k > 1 ? k * (unsigned long long)n_t : 0;
             // stored as int32; the host rejects the plan if a total exceeds 2^31 - 1
@@ -401,9 +408,9 @@ __global__ void k_units_gen(int B, int tile, long long smax, const int32_t *coun
         const int cnt = count[off + t];
         if (cnt == 0) continue;
         const long long ns = nsrc[t];
-        const int k = ns > smax ? (int)((ns + smax - 1) / smax) : 1;
         const int ntile = (cnt + tile - 1) / tile;
         const int l0 = sptr[t], l1 = sptr[t + 1];
+        const int k = p2p_segments((unsigned long long)ns, smax, l1 - l0);
         // emits segment j = [e_lo, e_hi) holding w sources (lanes over its tiles)
         auto emit = [&](int j, int e_lo, int e_hi, long long w) {
             for (int ti = lane; ti < ntile; ti += 32) {
@@ -556,7 +563,10 @@ std::atomic<long long> g_list_capacity{0x7fffffffLL};
 // Sources per near-field unit (about). A leaf's whole list up to
 // kP2PSegSources where the leaves' tiles alone give every SM kP2PUnitsPerSM
 // units; fewer leaves are cut into as many segments as make up that number,
-// down to kP2PSegMin sources (below, a unit's set-up outweighs its pairs).
+// down to kP2PSegMin sources (below, a unit's set-up outweighs its pairs) and to
+// whole source leaves (a list is cut between its entries: a tree of a few large
+// leaves stays at that many segments a leaf, and a heavy entry takes up several
+// segments' share).
 // 64 leaves of 78 points, every list the whole set: 225 us as 64 units, 43 us
 // as 1280. From 10 units per SM on, whole lists cost no more (the units go
 // heaviest first). 8 leaves of 125 points: 20.4 us with segments of 256

@@ -64,3 +64,21 @@ def test_clustered_set_splits_only_heavy_leaves(gpu_lib):
     assert fmm.fmm_plan_stats(p64)["p2p_partial_slots"] > 0
     g64, _ = fmm.fmm_eval(p64, qd.double())
     parity.check("split_fp64_gmm", "l2_phi", parity.rel_l2(g64.cpu().numpy()[t], op), 1e-6)
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("n,levels", [(1000, 0), (777, 0), (5000, 1), (3000, 2)])
+def test_no_more_segments_than_list_entries(gpu_lib, prec, n, levels):
+    """Trees of one or a few leaves: a strong list is cut between its entries, so a
+    leaf has no more segments than entries, and one of a single entry no partial sums.
+    theta = 0: the exact sum, to the bounds held above."""
+    fmm = gpu_lib
+    x, q = inputs.points("uniform", n, seed=n), inputs.charges_uniform(n, seed=n)
+    plan = fmm.fmm_plan(torch.from_numpy(x).cuda(), levels, 4, 0.0, prec=prec)
+    st = fmm.fmm_plan_stats(plan)
+    nl = 1 << levels
+    tiles = sum(-(-c // (32 if prec == 0 else 128)) for c in fmm.fmm_plan_tree(plan)["count"][nl - 1:])
+    assert st["p2p_units"] <= tiles * nl
+    assert st["p2p_partial_slots"] <= (n * nl if levels else 0)
+    pot = fmm.fmm_eval(plan, torch.from_numpy(q).cuda())[0].cpu().numpy()
+    assert parity.rel_l2(pot, oracle.direct(x, q)[0]) <= (1e-13 if prec == 0 else 1e-6)
