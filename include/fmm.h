@@ -445,13 +445,15 @@ int64_t fmm_set_list_capacity(int64_t entries);
 
 /*
  * fmm_set_wait_limit -- the bound of the device-side waits of the one-launch
- * downward pass (a box waits for its parent's expansion): `sleeps` waits of
- * ~0.1 us each before the wait gives up and the evaluation reports
- * FMM_ETIMEDOUT through fmm_eval_check (default and any value <= 0: 2^24,
- * ~2 s). `withhold` > 0 names a box (heap index) whose completion is never
- * signalled, so that its children's waits run out: a test of the timeout
- * path that needs no device fault (<= 0: none). Process-wide; returns the
- * previous limit.
+ * downward pass (a box waits for its parent's expansion) and of the mixed
+ * form's M2L up to order 12 (a warp waits for the copies of its source rows):
+ * `sleeps` waits of ~0.1 us each before the wait gives up and the evaluation
+ * reports FMM_ETIMEDOUT through fmm_eval_check (default and any value <= 0:
+ * 2^24, ~2 s). For tests of the timeout path that need no device fault,
+ * `withhold` > 0 names a box (heap index) whose completion the downward pass
+ * never signals, so that its children's waits run out, and `withhold` = -b < -1
+ * a box b whose row the M2L never copies (-1, 0: none). Process-wide; returns
+ * the previous limit.
  */
 int64_t fmm_set_wait_limit(int64_t sleeps, int64_t withhold);
 

@@ -407,8 +407,9 @@ def fmm_measure_peak(kind: str, iters: int = 1 << 16, stream=None):
 
 
 def fmm_set_wait_limit(sleeps: int, withhold: int = -1) -> int:
-    """Bound of the downward pass's device waits (sleeps of ~0.1 us; <= 0:
-    default) and, for tests, a box whose completion is never signalled."""
+    """Bound of the device waits of the downward pass and the float M2L (sleeps
+    of ~0.1 us; <= 0: default) and, for tests, a box whose completion is never
+    signalled (b > 0) or whose row the M2L never copies (-b < -1)."""
     return int(load().fmm_set_wait_limit(int(sleeps), int(withhold)))
 
 

@@ -1336,6 +1336,7 @@ cudaError_t m2l_external(Plan &P, int level, int64_t n, const int32_t *tgt, cons
 // (tests only; -1 = none). Set by fmm_set_wait_limit.
 std::atomic<long long> g_wait_limit{1LL << 24};
 std::atomic<long long> g_withhold{-1};
+std::atomic<int> g_withhold_copy{-1};  // box whose row the float M2L does not copy
 
 // the upward pass of binary levels in one launch, translations up to level `stop`
 void m2m_up(Plan &P, int stop) {
@@ -2236,7 +2237,8 @@ cudaError_t m2l_f32_all(Plan &P) {
     } else if (m2l_in_registers(P.p)) {
         const PairTable PT = pair_table(P);
         e = with_reg_order(P.p, [&](auto o) {
-            reg::reg_launch<decltype(o)::value>(PT, tot, P.box_cf, P.Mf, P.Lh, P.d_err, P.stream);
+            reg::reg_launch<decltype(o)::value>(PT, tot, P.box_cf, P.Mf, P.Lh, P.d_err,
+                                                 reg::Waits{g_wait_limit.load(), g_withhold_copy.load()}, P.stream);
             return cudaGetLastError();
         });
     } else {
@@ -2265,7 +2267,8 @@ cudaError_t batch_m2l(const BatchSys *S, const int32_t *off, int nsys, int64_t n
     if (nchunks == 0) return cudaGetLastError();
     if (m2l_in_registers(p))
         return with_reg_order(p, [&](auto o) {
-            reg::reg_launch_batch<decltype(o)::value>(S, off, nsys, nchunks, st);
+            reg::reg_launch_batch<decltype(o)::value>(S, off, nsys, nchunks,
+                                                       reg::Waits{g_wait_limit.load(), g_withhold_copy.load()}, st);
             return cudaGetLastError();
         });
     switch (p) {
@@ -2298,5 +2301,6 @@ extern "C" int64_t fmm_set_wait_limit(int64_t sleeps, int64_t withhold) {
     const long long prev = fmm::g_wait_limit.load();
     fmm::g_wait_limit.store(sleeps > 0 ? sleeps : (1LL << 24));
     fmm::g_withhold.store(withhold > 0 ? withhold : -1);
+    fmm::g_withhold_copy.store(withhold < -1 && withhold >= -0x7fffffffLL ? (int)-withhold : -1);
     return (int64_t)prev;
 }

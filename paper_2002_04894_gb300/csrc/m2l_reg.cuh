@@ -171,9 +171,11 @@ __device__ __forceinline__ float4 ld4(const void *p) {
 // The lanes' source rows, counted on the warp's mbarrier: one bulk copy for
 // each run of consecutive boxes (a target's sources ascend and siblings come
 // together). A copy's operands are warp-uniform registers, so every copy is a
-// trip of a loop: fewer copies, fewer instructions.
+// trip of a loop: fewer copies, fewer instructions. (withhold >= 0, tests only:
+// the run that holds this box is left out, and the wait for it runs out.)
 template <int P>
-__device__ __forceinline__ void copy_rows(const float2 *__restrict__ Mf, int gs, const char *row, uint32_t bar) {
+__device__ __forceinline__ void copy_rows(const float2 *__restrict__ Mf, int gs, const char *row, uint32_t bar,
+                                          int withhold) {
     const int lane = threadIdx.x & 31;
     const int prev = __shfl_up_sync(0xffffffffu, gs, 1);
     const bool head = lane == 0 || gs != prev + 1;
@@ -183,7 +185,7 @@ __device__ __forceinline__ void copy_rows(const float2 *__restrict__ Mf, int gs,
         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(32 * row_bytes(P))
                      : "memory");
     __syncwarp();
-    if (head)
+    if (head && !(withhold >= gs && withhold < gs + len))
         asm volatile(
             "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
                 (uint32_t)__cvta_generic_to_shared(row)),
@@ -191,12 +193,12 @@ __device__ __forceinline__ void copy_rows(const float2 *__restrict__ Mf, int gs,
             : "memory");
 }
 
-// Waits for phase `parity` of the warp's copies, a bounded number of tries
-// (each suspends for a while in hardware; a copy takes microseconds). False
-// if the bound ran out.
-__device__ __forceinline__ bool wait_rows(uint32_t bar, uint32_t parity) {
-    for (int i = 0; i < (1 << 16); i++) {
-        uint32_t ok;
+// Waits for phase `parity` of the warp's copies: a few tries that suspend in
+// hardware (a copy takes microseconds), then `limit` sleeps of ~0.1 us. False if
+// the bound ran out.
+__device__ __forceinline__ bool wait_rows(uint32_t bar, uint32_t parity, long long limit) {
+    uint32_t ok = 0;
+    for (int i = 0; i < 8; i++) {
         asm volatile(
             "{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
             : "=r"(ok)
@@ -204,8 +206,23 @@ __device__ __forceinline__ bool wait_rows(uint32_t bar, uint32_t parity) {
             : "memory");
         if (ok) return true;
     }
+    for (long long i = 0; i < limit; i++) {
+        __nanosleep(100);
+        asm volatile(
+            "{ .reg .pred p; mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
+            : "=r"(ok)
+            : "r"(bar), "r"(parity)
+            : "memory");
+        if (ok) return true;
+    }
     return false;
 }
+
+// the waits' bound and the box whose row is not copied (-1: none), as set by fmm_set_wait_limit
+struct Waits {
+    long long limit;
+    int withhold;
+};
 
 // degree N of this lane's row, two coefficients per 16-byte read where the pair is aligned
 template <int N>
@@ -447,7 +464,7 @@ struct Batched {
 // The next chunk's source rows are copied to shared memory while this one is
 // translated and rotated back.
 template <int P, typename Src>
-__device__ __forceinline__ void run(Src &src, char *slice) {
+__device__ __forceinline__ void run(Src &src, char *slice, const Waits &wt) {
     const unsigned W = blockDim.x >> 5, total = src.chunks(), stride = gridDim.x * W;
     unsigned w0 = blockIdx.x * W;  // the block's first chunk (device memory holds fewer than 2^31 chunks of pairs)
     if (w0 >= total) return;
@@ -468,7 +485,7 @@ __device__ __forceinline__ void run(Src &src, char *slice) {
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncwarp();
-    copy_rows<P>(src.Mf(nxt), nxt.gs, rowp, bar);
+    copy_rows<P>(src.Mf(nxt), nxt.gs, rowp, bar, wt.withhold);
     uint32_t parity = 0;
     bool lost = false;  // a wait ran out (lanes of a warp agree: they test the same barrier phase)
     for (;; w0 += stride) {
@@ -484,7 +501,7 @@ __device__ __forceinline__ void run(Src &src, char *slice) {
         const float2 eb = make_float2(dz * rinv, rxy * rinv);
         const float2 eai = make_float2(ea.y, -ea.x);  // -i e^{ia}
         const float qs = (sh.w > 0.f ? sh.w : 1.f) * rinv, qt = (th.w > 0.f ? th.w : 1.f) * rinv;
-        if (!lost && !wait_rows(bar, parity)) {
+        if (!lost && !wait_rows(bar, parity, wt.limit)) {
             lost = true;  // no more copies; the warp goes on, for the block's barriers (FMM_ETIMEDOUT: results invalid)
             atomicOr(src.err(cur) + 1, 16);
         }
@@ -514,7 +531,7 @@ __device__ __forceinline__ void run(Src &src, char *slice) {
             if constexpr (P - L >= sync_from<P>()) __syncthreads();
             axial<P, L>(S);
             if constexpr (L == P / 6) {
-                if (more && !__any_sync(0xffffffffu, lost)) copy_rows<P>(src.Mf(nxt), nxt.gs, rowp, bar);
+                if (more && !__any_sync(0xffffffffu, lost)) copy_rows<P>(src.Mf(nxt), nxt.gs, rowp, bar, wt.withhold);
             }
         });
         {
@@ -536,24 +553,24 @@ __device__ __forceinline__ void run(Src &src, char *slice) {
         }
         if (!more) break;
     }
-    if (lost) wait_rows(bar, parity);  // its copies still in flight
+    if (lost) wait_rows(bar, parity, wt.limit);  // its copies still in flight
 }
 
 template <int P>
 __global__ void __launch_bounds__(warps<P>() * 32, 1)
 k_m2l_reg(PairTable PT, const float4 *__restrict__ cf, const float2 *__restrict__ Mf, double2 *__restrict__ Lh,
-          int *err) {
+          int *err, Waits wt) {
     extern __shared__ float4 sm4[];
     OnePlan src{PT, cf, Mf, Lh, err, PT.lmin};
-    run<P>(src, (char *)sm4 + (threadIdx.x >> 5) * slice_bytes<P>());
+    run<P>(src, (char *)sm4 + (threadIdx.x >> 5) * slice_bytes<P>(), wt);
 }
 
 template <int P>
 __global__ void __launch_bounds__(warps<P>() * 32, 1)
-k_b_m2l_reg(const BatchSys *__restrict__ S, const int32_t *__restrict__ off, int nsys) {
+k_b_m2l_reg(const BatchSys *__restrict__ S, const int32_t *__restrict__ off, int nsys, Waits wt) {
     extern __shared__ float4 sm4[];
     Batched src{S, off, nsys};
-    run<P>(src, (char *)sm4 + (threadIdx.x >> 5) * slice_bytes<P>());
+    run<P>(src, (char *)sm4 + (threadIdx.x >> 5) * slice_bytes<P>(), wt);
 }
 
 template <int P>
@@ -568,20 +585,20 @@ unsigned grid(int64_t warp_chunks) {
 }
 template <int P>
 void reg_launch(const PairTable &PT, int64_t tot, const float4 *cf, const float2 *Mf, double2 *Lh, int *err,
-                cudaStream_t st) {
-    FMM_LAUNCH(k_m2l_reg<P>, grid<P>((tot + 31) / 32), warps<P>() * 32, smem_bytes<P>(), st, PT, cf, Mf, Lh, err);
+                Waits wt, cudaStream_t st) {
+    FMM_LAUNCH(k_m2l_reg<P>, grid<P>((tot + 31) / 32), warps<P>() * 32, smem_bytes<P>(), st, PT, cf, Mf, Lh, err, wt);
 }
 template <int P>
-void reg_launch_batch(const BatchSys *S, const int32_t *off, int nsys, int64_t nchunks, cudaStream_t st) {
-    FMM_LAUNCH(k_b_m2l_reg<P>, grid<P>(nchunks * 4), warps<P>() * 32, smem_bytes<P>(), st, S, off, nsys);
+void reg_launch_batch(const BatchSys *S, const int32_t *off, int nsys, int64_t nchunks, Waits wt, cudaStream_t st) {
+    FMM_LAUNCH(k_b_m2l_reg<P>, grid<P>(nchunks * 4), warps<P>() * 32, smem_bytes<P>(), st, S, off, nsys, wt);
 }
 
 // explicit instances of one order (each translation unit holds a few: they compile in parallel)
 #define FMM_M2L_REG(PRE, P)                                                                                   \
     PRE template cudaError_t reg_attr<P>();                                                                   \
     PRE template void reg_launch<P>(const PairTable &, int64_t, const float4 *, const float2 *, double2 *,    \
-                                    int *, cudaStream_t);                                                            \
-    PRE template void reg_launch_batch<P>(const BatchSys *, const int32_t *, int, int64_t, cudaStream_t);
+                                    int *, Waits, cudaStream_t);                                              \
+    PRE template void reg_launch_batch<P>(const BatchSys *, const int32_t *, int, int64_t, Waits, cudaStream_t);
 
 }  // namespace reg
 }  // namespace fmm

@@ -135,3 +135,41 @@ def test_downward_wait_that_runs_out_reports_etimedout(gpu_lib):
     again, _ = fmm.fmm_eval(plan2, q)
     fmm.fmm_eval_check(plan2)
     assert (torch.linalg.norm(again - good) / torch.linalg.norm(good)).item() <= 1e-13
+
+
+@pytest.mark.parametrize("batched", [False, True])
+@pytest.mark.parametrize("p", [4, 9, 12])
+def test_m2l_wait_that_runs_out_reports_etimedout(gpu_lib, p, batched):
+    """The float M2L waits (bounded) for its warps' copies of source rows. A row
+    that is never copied (test hook) makes the wait run out: the evaluation ends, and
+    fmm_eval_check reports FMM_ETIMEDOUT. With the limit restored a new plan evaluates
+    as before (the same sums in another order of the double atomics)."""
+    fmm = gpu_lib
+    x = torch.from_numpy(inputs.points("uniform", 20000, 4)).cuda()
+    q = torch.from_numpy(inputs.charges_uniform(20000, 4)).cuda()
+    B = 8
+
+    def evaluate():
+        plan = fmm.fmm_plan(x, B, p, 0.5, prec=fmm.FMM_PREC_MIXED)
+        if not batched:
+            return plan, fmm.fmm_eval(plan, q)[0], None
+        pot = torch.empty_like(q)
+        torch.cuda.synchronize()
+        batch = fmm.fmm_batch_create([plan], [q], [pot])
+        fmm.fmm_batch_launch(batch)
+        return plan, pot, batch
+
+    plan, good, batch = evaluate()
+    fmm.fmm_eval_check(plan)
+    prev = fmm.fmm_set_wait_limit(2000, -((1 << B) - 1))     # the first leaf's row
+    try:
+        plan, _, batch = evaluate()
+        with pytest.raises(fmm.FmmError) as e:
+            fmm.fmm_eval_check(plan)
+        assert e.value.status == -5        # FMM_ETIMEDOUT
+    finally:
+        fmm.fmm_set_wait_limit(0, -1)
+    assert prev > 0
+    plan, again, batch = evaluate()
+    fmm.fmm_eval_check(plan)
+    assert (torch.linalg.norm(again - good) / torch.linalg.norm(good)).item() <= 1e-6
