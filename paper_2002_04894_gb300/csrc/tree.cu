@@ -476,8 +476,8 @@ k_split_cluster(int level, const double *__restrict__ xin, const double *__restr
         }
         __syncthreads();
         if (s_one && pass < 7) {  // one key under the prefix: its CTA tells the others
-            cl.sync();            // every CTA has written its own prefix
             const uint64_t pre2 = s_prefix;
+            cl.sync();  // every CTA has written and read its own prefix
             for (int i = tid; i < m; i += kClThreads) {
                 const uint64_t kk = keys[i];
                 if ((kk >> shift) == (pre2 >> shift))
