@@ -290,7 +290,7 @@ k_p2p_tf(int B, int64_t n, const double *__restrict__ x, const double *__restric
 // targets 0.38 -> 0.08.
 // ---------------------------------------------------------------------------
 constexpr int kRec = 7;
-constexpr int kFlush = 1024;  // records between flushes: three-float sums of 1000 terms hold 2^-57 of them, of 10^6 2^-51
+constexpr int kFlush = 1024;  // records between flushes: three-float sums of 1000 terms lose less than 2^-55 of them, of 10^6 2^-51
 constexpr int64_t kSlab = 1 << 20;  // sources split at a time (58 MB of records)
 
 // the grid of the points: centre, 2^-k, whether it holds (grid_exponent), and the charges' exponent
