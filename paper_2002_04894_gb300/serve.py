@@ -68,13 +68,16 @@ def default_levels(n: int, leaf: float = 100.0) -> int:
 
 def plan_bytes(n: int, levels: int, p: int, mixed: bool = True) -> int:
     """Upper estimate of a plan's device memory while it is built and used:
-    points, boxes, lists and expansions (persistent) plus the build's
-    temporaries, plus the caller's input and output copies."""
+    points (the FP64 form's also as three floats), boxes, lists and expansions
+    (persistent) plus the build's temporaries, plus the caller's input and
+    output copies. Lists of strongly clustered points can exceed it."""
     nbox = (2 << levels) - 1
     nleaf = 1 << levels
     nc = (p + 1) * (p + 2) // 2
-    persist = n * (96 + (60 if mixed else 0)) + nbox * (128 + 32 * nc + (24 * nc if mixed else 0))
-    lists = nleaf * 3000
+    persist = n * (96 + (60 if mixed else 56)) + nbox * (128 + 32 * nc + (24 * nc if mixed else 0))
+    # few leaves: the near field's partial sums (32 bytes each), 10 units of 128 targets for each of 152 SMs
+    split = 32 * (10 * 152 * 128 + 2 * n) if n < 10 * 152 * 128 else 0
+    lists = nleaf * 3000 + split
     scratch = n * 40 + nbox * 64 + nleaf * 2000
     io = n * 8 * 8
     return int(1.25 * (persist + lists + scratch + io)) + (4 << 20)

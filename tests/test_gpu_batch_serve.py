@@ -235,6 +235,41 @@ def test_tuner_times_the_evaluation_that_will_run(gpu_lib, monkeypatch, batch, f
     assert set(asked) == {fields is not False}
 
 
+@pytest.mark.parametrize("p", [7, 12])
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("n", [1000, 5000, 20000, 100_000, 1_000_000])
+def test_plan_bytes_covers_the_plan(gpu_lib, n, prec, p):
+    """What the server reserves for a request is at least what its plan takes from
+    the allocator at its peak, with the request's inputs and outputs."""
+    import ctypes as C
+    fmm = gpu_lib
+    live, peak = {}, [0]
+
+    def alloc(nbytes, ctx, stream):
+        ptr = torch.cuda.caching_allocator_alloc(int(nbytes), torch.cuda.current_device(), int(stream or 0))
+        live[ptr] = int(nbytes)
+        peak[0] = max(peak[0], sum(live.values()))
+        return ptr
+
+    def free(ptr, nbytes, ctx, stream):
+        del live[ptr]
+        torch.cuda.caching_allocator_delete(ptr)
+
+    cb = fmm.ALLOC_FN(alloc), fmm.FREE_FN(free)
+    levels = serve.default_levels(n)
+    x = torch.from_numpy(inputs.points("uniform", n, 1)).cuda()
+    q, pot, fld = torch.ones(n, 5, dtype=torch.float64, device="cuda").split([1, 1, 3], 1)
+    q, pot, fld = q.contiguous(), pot.contiguous(), fld.contiguous()
+    h, st = C.c_void_p(), torch.cuda.current_stream().cuda_stream
+    assert fmm.fmm_plan_raw(fmm.load(), x.data_ptr(), n, 0, fmm.fmm_opts(levels, p, 0.5, prec, 0, 1.0, 1),
+                            fmm.fmm_allocator(*cb, None), st, h) == 0
+    assert fmm.load().fmm_eval(h, q.data_ptr(), pot.data_ptr(), fld.data_ptr(), st) == 0
+    torch.cuda.synchronize()
+    fmm.load().fmm_destroy(h)
+    assert not live
+    assert peak[0] + 64 * n <= serve.plan_bytes(n, levels, p, prec == 1)
+
+
 def test_server_resident_plans_equal_fresh_solves(gpu_lib):
     """Requests naming their point set (geom) reuse a resident plan with new
     charges: each result equals a fresh solve of the same points and charges,
