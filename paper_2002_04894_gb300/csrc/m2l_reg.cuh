@@ -15,9 +15,9 @@
 // registers), over 60% busy, with the straight-line code (120 KB at p = 12)
 // read through the instruction caches, and the 32-lane sums into the targets
 // (0.9 of 5.4 ms). 1.62e7 pairs of 2M Plummer points, 14 levels, M2L stage
-// before and now: p = 12 10.74 -> 5.05 ms, p = 10 6.91 -> 3.32, p = 8 4.39 ->
-// 1.72, p = 4 1.64 -> 0.52; odd orders (formerly tensor-core products) p = 9
-// 81.5 -> 2.65.
+// before and now: p = 12 10.74 -> 5.18 ms, p = 10 6.91 -> 3.40, p = 8 4.39 ->
+// 1.75, p = 4 1.64 -> 0.55; odd orders (formerly tensor-core products) p = 9
+// 81.5 -> 2.75.
 #pragma once
 
 #include <algorithm>
@@ -249,7 +249,7 @@ __device__ __forceinline__ void read_deg(const char *row, float (&r)[N + 1], flo
 // fetched once per SM and pass, not once per warp. Measured on 1.62e7 pairs
 // with barriers from degree 4 on / P - 2 / P - 1 / none: p = 12 5.36 / 5.05 /
 // 5.13 / 5.36 ms, p = 10 3.52 / 3.43 / 3.32 / 3.38, p = 8 2.01 / 1.97 / 1.85 /
-// 1.72, p = 6 1.25 / 1.22 / 1.14 / 0.91: the code of the orders below 10 fits
+// 1.72, p = 6 1.25 / 1.22 / 1.14 / 0.91 (with weighted sums): the code of the orders below 10 fits
 // the instruction cache and the barriers only cost.
 template <int P>
 constexpr int sync_from() { return P >= 12 ? P - 2 : P >= 10 ? P - 1 : P + 1; }
@@ -315,7 +315,9 @@ __host__ __device__ constexpr int group_first(int n) {  // first degree of degre
 // the run's target's scaled local in double. mask: of several runs, the lanes
 // of the present one as bits all 1, the others 0, so that a warp with several
 // targets costs a pass per run and not a loop over its lanes. (Bits and not
-// weights of 0 and 1: another target's sum may hold an infinity.)
+// weights of 0 and 1: another target's sum may hold an infinity. p = 12 5.18 ms
+// against 5.10 with weights; weights, and the sums that come out not finite
+// formed again, 5.33; loops over a run's quads 5.46.)
 template <int P, int G, int N>
 __device__ __forceinline__ void sum_group(const float *red, uint32_t *mask, int t32, unsigned ends,
                                           double2 *__restrict__ Lh) {

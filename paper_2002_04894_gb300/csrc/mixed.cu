@@ -675,7 +675,8 @@ __device__ __forceinline__ void p2p_f32_body(int B, int64_t n, const float *__re
 // 128-target tiles (8 blocks) and 80 for 64-target tiles (12 blocks) the
 // 512-system batch ran in 319.0 ms, against 324.8 ms at 80 registers for both
 // (328 ms at 72); since the tiles' last targets share threads, 9 blocks (56
-// registers): 48 systems 18.25 -> 17.93 ms (10 blocks 18.21). The single-plan kernel takes 8 blocks for 128-target tiles
+// registers): 48 systems 18.25 -> 17.93 ms (10 blocks 18.21), 512 systems 278.9 ->
+// 276.2. The single-plan kernel takes 8 blocks for 128-target tiles
 // (16.4 ms on 2M points; 16.9 with 7) and is left unconstrained for 64-target
 // tiles (61.2 ms on 8M points at 96 registers; 61.7 with 14 blocks).
 template <int T>

@@ -18,7 +18,10 @@
 // bits) is rounded to it and marked; a pair goes through FP64 arithmetic on the
 // original doubles instead when its distance is below 2^-19 of the extent
 // with a marked point, below 2^-23 otherwise (that includes r = 0), or when
-// the charge is not finite or below 2^-60 of the largest.
+// the charge is not finite or below 2^-60 of the largest. Such a pair costs
+// both arithmetics: 200k Plummer points with one more at 1e5 of their size
+// 121 ms, at 1e6 (all near pairs left to FP64) 447, charges over 24 decades
+// 145, over 40 245; FP64 arithmetic alone 563 to 581 (whole evaluations).
 
 #include <algorithm>
 #include <type_traits>

@@ -14,7 +14,8 @@
 // A pair whose positions are exact on the common grid has relative errors of
 // at most 2^-61 (potential) and 2^-58 (field) over 1.6 million random pairs at
 // distances from 1 to 1e-7 of the grid's extent (double arithmetic: 2^-51 and
-// 2^-50); close pairs of rounded positions are left to FP64 (p2p_tf.cu).
+// 2^-50); close pairs of rounded positions are left to FP64 (p2p_tf.cu). The
+// host branch below is for tests/test_trifloat_cpu.py, which holds these bounds.
 #pragma once
 
 #ifndef __CUDACC__
